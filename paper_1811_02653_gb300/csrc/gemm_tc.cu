@@ -40,6 +40,8 @@ using namespace tc;
 
 constexpr int BM = 128;
 constexpr int ROWB = 128;                     // bytes per tile row: one 128-byte swizzle row
+constexpr int kEpiPitch = 33;                 // words per row of an epilogue warp's 32 x 32 piece
+constexpr size_t kEpiBytes = 4 * 32 * kEpiPitch * sizeof(float);   // the four epilogue warps
 
 // Operand kinds.  Bf16: BF16 operands, 64 K-elements per 128-byte stage row,
 // tcgen05 kind::f16.  Tf32x3: FP32 operands given as two TF32-exact planes
@@ -74,7 +76,7 @@ struct Cfg {
     static constexpr int ACC_STRIDE = FP8 ? 256 : BN;
     static constexpr int TMEM_COLS = FP8 ? 512 : 2 * BN;
     static constexpr int SF_GAP_SLOTS = (256 - BN) / 16;
-    static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 256;
+    static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 256 + kEpiBytes;
     // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue; FP8 adds warp 6, which turns
     // each stage's FP32 scales into UE8M0 chunks ahead of the MMA warp
     static constexpr int THREADS = FP8 ? 224 : 192;
@@ -151,6 +153,55 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
     const int in = t - group * G * tiles_n;
     tm = first_m + in % gm;
     tn = in / gm;
+}
+
+// Write-out of one 32 x 32 piece of an accumulator by one warp: lane i holds row
+// r0 + i, columns cb .. cb+31, in v.  The piece goes through the warp's own 32 x 33
+// words of shared memory so that the warp's stores cover whole 128-byte row
+// pieces of C.  Stored straight from the registers (one row per lane) every
+// instruction touches 32 lines, and nothing hides that when a CTA has a single
+// tile: on GB300 the 2003 x 1777 x 3840 BF16 product (scalar stores: ldc is odd)
+// took 47.6 us that way and takes 32.7, 1024 x 1501 x 2048 35.7 -> 22.8, the
+// grouped launch of 16 uneven products 861 -> 779, the FP8 product of 8192^3
+// (16-byte stores, beside the next tile's MMAs) 514 -> 472.
+// The odd pitch keeps both the column writes and the row reads free of conflicts.
+__device__ __forceinline__ void store_piece(float *buf, const float *v, float alpha, float beta, float *C,
+                                            int64_t ldc, int64_t r0, int64_t m, int64_t cb, int64_t l, bool vec_ok,
+                                            int lane) {
+    __syncwarp();   // the previous piece has been read
+#pragma unroll
+    for (int u = 0; u < 32; ++u) buf[lane * kEpiPitch + u] = alpha * v[u];
+    __syncwarp();
+    if (vec_ok && cb + 32 <= l) {
+        // 4 rows per instruction, 8 lanes of 16 bytes each
+        const int rr = lane >> 3, cc = (lane & 7) * 4;
+        float *dst = C + (r0 + rr) * ldc + cb + cc;
+#pragma unroll
+        for (int t = 0; t < 8; ++t, dst += 4 * ldc) {
+            const float *src = buf + (4 * t + rr) * kEpiPitch + cc;
+            float4 o = make_float4(src[0], src[1], src[2], src[3]);
+            if (r0 + 4 * t + rr < m) {
+                if (beta != 0.f) {
+                    const float4 old = *reinterpret_cast<const float4 *>(dst);
+                    o.x = fmaf(beta, old.x, o.x);
+                    o.y = fmaf(beta, old.y, o.y);
+                    o.z = fmaf(beta, old.z, o.z);
+                    o.w = fmaf(beta, old.w, o.w);
+                }
+                *reinterpret_cast<float4 *>(dst) = o;
+            }
+        }
+    } else if (cb + lane < l) {
+        float *dst = C + r0 * ldc + cb + lane;
+#pragma unroll 8
+        for (int t = 0; t < 32; ++t, dst += ldc) {
+            if (r0 + t < m) {
+                float o = buf[t * kEpiPitch + lane];
+                if (beta != 0.f) o = fmaf(beta, *dst, o);
+                *dst = o;
+            }
+        }
+    }
 }
 
 // Product owning global tile t of a grouped launch: the last p with begin[p] <= t.
@@ -469,43 +520,17 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
     } else {
         // ---------------- epilogue (warps 2..5) ----------------
         const int quarter = warp & 3;                 // TMEM lanes 32*quarter .. +31
-        const int row_in_tile = quarter * 32 + lane;
+        float *buf = reinterpret_cast<float *>(smem + STAGES * C::STAGE_BYTES + 256) + quarter * 32 * kEpiPitch;
         int iter = 0;
-        // FP32 store of 32 consecutive values of row r starting at column cbase
-        auto store32 = [&](const TileJob &j, bool vec_ok, int64_t r, int64_t cbase, const float *val) {
-            if (r >= j.m) return;
-            float *dst = j.C + r * j.ldc + cbase;
-            if (vec_ok && cbase + 32 <= j.l) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    float4 o = make_float4(j.alpha * val[4 * u + 0], j.alpha * val[4 * u + 1],
-                                           j.alpha * val[4 * u + 2], j.alpha * val[4 * u + 3]);
-                    if (j.beta != 0.f) {
-                        const float4 old = *reinterpret_cast<const float4 *>(dst + 4 * u);
-                        o.x = fmaf(j.beta, old.x, o.x);
-                        o.y = fmaf(j.beta, old.y, o.y);
-                        o.z = fmaf(j.beta, old.z, o.z);
-                        o.w = fmaf(j.beta, old.w, o.w);
-                    }
-                    *reinterpret_cast<float4 *>(dst + 4 * u) = o;
-                }
-            } else {
-#pragma unroll
-                for (int u = 0; u < 32; ++u) {
-                    if (cbase + u < j.l) {
-                        float o = j.alpha * val[u];
-                        if (j.beta != 0.f) o = fmaf(j.beta, dst[u], o);
-                        dst[u] = o;
-                    }
-                }
-            }
-        };
         bool ok = true;
         for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
             const TileJob j = job(t);
             const bool vec_ok = ((reinterpret_cast<uintptr_t>(j.C) & 15u) == 0) && (j.ldc % 4 == 0);
-            const int64_t r = (int64_t)j.tm * BM + row_in_tile;
+            const int64_t r0 = (int64_t)j.tm * BM + quarter * 32;
             const int64_t c0 = (int64_t)j.tn * BN;
+            auto store = [&](int ch, const float *val) {
+                store_piece(buf, val, j.alpha, j.beta, j.C, j.ldc, r0, j.m, c0 + ch * 32, j.l, vec_ok, lane);
+            };
             if constexpr (C::CHUNK_KB < (1 << 30)) {
                 // chunked accumulation: running FP32 sum of the tile row in registers
                 float total[BN];
@@ -530,7 +555,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                 }
                 if (!ok) break;
 #pragma unroll
-                for (int ch = 0; ch < BN / 32; ++ch) store32(j, vec_ok, r, c0 + ch * 32, total + ch * 32);
+                for (int ch = 0; ch < BN / 32; ++ch) store(ch, total + ch * 32);
             } else {
                 const int a = iter & 1;
                 const uint32_t aphase = (uint32_t)(iter >> 1) & 1u;
@@ -546,7 +571,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
 #pragma unroll
                         for (int u = 0; u < 32; ++u) v[u] = 0u;   // no kept block: a zero product
                     }
-                    store32(j, vec_ok, r, c0 + ch * 32, reinterpret_cast<const float *>(v));
+                    store(ch, reinterpret_cast<const float *>(v));
                 }
                 tc_fence_before();
                 mbar_arrive(&tmem_empty[a]);
@@ -585,7 +610,7 @@ struct CfgPair {
     static constexpr uint32_t PAIR_TX = 2u * STAGE_BYTES;   // both CTAs' loads land on the leader's barrier
     static constexpr int TMEM_COLS = 512;             // two 256-column accumulators
     static constexpr int THREADS = 192;
-    static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 256;
+    static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 256 + kEpiBytes;
     static constexpr uint32_t IDESC = idesc_bf16_f32(2 * BM, BN);
     static_assert(SMEM <= 232448, "shared memory");
 };
@@ -778,6 +803,7 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
         // ---------------- epilogue (warps 2..5): this CTA's 128 rows ----------------
         const int quarter = warp & 3;
         const int row_in_tile = quarter * 32 + lane;
+        float *buf = reinterpret_cast<float *>(smem + STAGES * C::STAGE_BYTES + 256) + quarter * 32 * kEpiPitch;
         const uint32_t empty_cl0 = cluster_addr(&tmem_empty[0], 0);
         const uint32_t empty_cl1 = cluster_addr(&tmem_empty[1], 0);
         int iter = 0;
@@ -802,35 +828,10 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
 #pragma unroll
                     for (int u = 0; u < 32; ++u) v[u] = 0u;
                 }
+                const int64_t cb = c0 + ch * 32;
+                store_piece(buf, reinterpret_cast<const float *>(v), alpha, g.beta, g.C, g.ldc, r - lane, g.m, cb, g.l,
+                            vec_ok, lane);
                 if (r < g.m) {
-                    float *dst = g.C + r * g.ldc + c0 + ch * 32;
-                    const int64_t cb = c0 + ch * 32;
-                    if (vec_ok && cb + 32 <= g.l) {
-#pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            float4 o = make_float4(alpha * __uint_as_float(v[4 * u]),
-                                                   alpha * __uint_as_float(v[4 * u + 1]),
-                                                   alpha * __uint_as_float(v[4 * u + 2]),
-                                                   alpha * __uint_as_float(v[4 * u + 3]));
-                            if (g.beta != 0.f) {
-                                const float4 old = *reinterpret_cast<const float4 *>(dst + 4 * u);
-                                o.x = fmaf(g.beta, old.x, o.x);
-                                o.y = fmaf(g.beta, old.y, o.y);
-                                o.z = fmaf(g.beta, old.z, o.z);
-                                o.w = fmaf(g.beta, old.w, o.w);
-                            }
-                            *reinterpret_cast<float4 *>(dst + 4 * u) = o;
-                        }
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < 32; ++u) {
-                            if (cb + u < g.l) {
-                                float o = alpha * __uint_as_float(v[u]);
-                                if (g.beta != 0.f) o = fmaf(g.beta, dst[u], o);
-                                dst[u] = o;
-                            }
-                        }
-                    }
                     if (g.sym && (tm >> 1) != tn) {
                         // the mirror tile: value (r, cb + u) also at (cb + u, r); the
                         // warp's 32 rows make each of these stores one 128-byte line

@@ -27,6 +27,8 @@ os_status sketch_left_sparse_impl(const Plan *p, const void *A, os_dtype a_t, in
 os_status gemm_masked_f32(const Plan *p, const float *At, int64_t ldat, const float *BtT,
                           int64_t ldbt, int64_t m, int64_t l, uint64_t mask, float alpha, float beta,
                           float *C, int64_t ldc, cudaStream_t st);
+os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &b, int64_t ld, int64_t l,
+                            uint64_t mask, float alpha, float *C, int64_t ldc, unsigned int *flag, cudaStream_t st);
 os_status gemm_bf16_mn(const void *A, int64_t lda, bool a_mn, const void *B, int64_t ldb, bool b_mn, int64_t m,
                        int64_t l, int64_t K, float alpha, float *C, int64_t ldc, int32_t mn_b, int32_t remap,
                        uint64_t mask, int32_t P, cudaStream_t st);
@@ -106,6 +108,37 @@ MatmulLayout layout(const Plan *p, int64_t m, int64_t l, os_dtype a_t, os_dtype 
     }
     L.left_ws = align256(wl > wr ? wl : wr);
     return L;
+}
+
+// Whether an FP32 product runs on FP16 planes (sketches as FP32 sums, split row by
+// row, gemm_masked_f16x3) instead of on TF32 planes written by the sketches: block
+// widths that fit the 64-element K tile, scratch space for the row scales, and a
+// GEMM that gains more than the split and its launches cost.  On GB300 a 128 x 128
+// tile of the 3xTF32 kernel takes 19.5 ns per K (152 at once), a 256 x 160 tile of
+// the FP16 one 10.2 ns (76 at once); the memory-bound split and the four extra
+// launches take 8 bytes per sum at 6 TB/s and about 20 us.  Whole products, TF32 ->
+// FP16: 8192 x 32768 x 8192 (K = 8192) 5.39 -> 3.57 ms, 4096 x 16384 x 4096 (4096)
+// 818 -> 604 us, 1024 x 16384 x 1024 (4096) 169 -> 165, and just below the line
+// 512 x 8192 x 512 (2048) 74 -> 80, 1024 x 8192 x 1024 (2048) 95 -> 107.
+bool f16x3_pays(const Plan *p, os_dtype gemm_dtype, int64_t m, int64_t l, uint64_t mask, size_t scratch) {
+    if (gemm_dtype != OS_F32 || p->b % 64 != 0) return false;
+    if (scratch < (size_t)(m + l) * 4 + 512) return false;
+    const double K = (double)__builtin_popcountll(mask) * p->b;
+    auto waves = [](int64_t tiles, int at_once) { return (double)((tiles + at_once - 1) / at_once); };
+    const double tf32 = waves((m + 127) / 128 * ((l + 127) / 128), 152) * K * 19.5e-3;   // us
+    const double f16 = waves((m + 255) / 256 * ((l + 159) / 160), 76) * K * 10.2e-3;
+    return tf32 - f16 > 20.0 + (double)(m + l) * K * 8.0 / 6e6;
+}
+
+// The masked product of FP32 sums stored as TF32 pairs are (sums, then a plane's
+// room), by f16x3_pays; scratch holds the row scales and the flag.
+os_status matmul_f16x3(const Plan *p, void *At, void *BtT, int64_t ld, int64_t m, int64_t l, uint64_t mask, float *C,
+                       int64_t ldc, void *scratch, cudaStream_t st) {
+    unsigned int *flag = reinterpret_cast<unsigned int *>((reinterpret_cast<uintptr_t>(scratch) + 255) & ~uintptr_t(255));
+    float *sa = reinterpret_cast<float *>(flag + 4);
+    const SplitSide a{reinterpret_cast<float *>(At), m, sa};
+    const SplitSide b{reinterpret_cast<float *>(BtT), BtT == At ? 0 : l, BtT == At ? sa : sa + m};
+    return gemm_masked_f16x3(p, a, b, ld, l, mask, 1.0f / (float)__builtin_popcountll(mask), C, ldc, flag, st);
 }
 
 // Deterministic FP64 partial sums: fixed grid, fixed per-thread order, fixed tree.
@@ -231,6 +264,8 @@ extern "C" os_status oversketch_matmul(oversketch_plan_t plan, const void *A, os
     if (!A || !C || (!sym && !B)) return OS_ERR_INVALID_ARG;
     const os_dtype g = sketch_dtype(p, g0);
     const MatmulLayout L = layout(p, m, l, a_t, b_t, opts);
+    const bool f16 = f16x3_pays(p, g0, m, l, mask, L.left_ws);
+    const os_dtype sk = f16 ? OS_F32 : g;   // what the sketches write
     const size_t need = L.at_bytes + L.bt_bytes + L.as_bytes + L.bs_bytes + L.left_ws + 256;
     if (!workspace || ws_bytes < need) return OS_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
@@ -245,10 +280,11 @@ extern "C" os_status oversketch_matmul(oversketch_plan_t plan, const void *A, os
     // Only the kept blocks are sketched: the dropped blocks' columns of A~ and
     // B~ would never be read by the masked GEMM.
     if (opts && (opts->flags & OS_OPT_SPARSE_A) && sketch_left_sparse_fits(p, mask))
-        OSK_TRY(sketch_left_sparse_impl(p, A, a_t, m, lda, At, g, L.ldat, as, cs, mask, st));
+        OSK_TRY(sketch_left_sparse_impl(p, A, a_t, m, lda, At, sk, L.ldat, as, cs, mask, st));
     else
-        OSK_TRY(sketch_left_impl(p, A, a_t, m, lda, At, g, L.ldat, as, cs, mask, lws, L.left_ws, st));
-    if (!sym) OSK_TRY(sketch_right_impl(p, B, b_t, l, ldb, BtT, g, L.ldbt, bs, mask, lws, L.left_ws, st));
+        OSK_TRY(sketch_left_impl(p, A, a_t, m, lda, At, sk, L.ldat, as, cs, mask, lws, L.left_ws, st));
+    if (!sym) OSK_TRY(sketch_right_impl(p, B, b_t, l, ldb, BtT, sk, L.ldbt, bs, mask, lws, L.left_ws, st));
+    if (f16) return matmul_f16x3(p, At, BtT, L.ldat, m, l, mask, C, ldc, lws, st);
     return oversketch_gemm_masked(plan, At, L.ldat, as, BtT, L.ldbt, bs, g, m, l, mask, 1.0f, 0.0f, C, ldc,
                                   stream);
 }
@@ -392,6 +428,8 @@ extern "C" os_status oversketch_matmul_host(oversketch_plan_t plan, const void *
     const size_t pack_bytes = h.mm_bytes - 256 - (L.at_bytes + L.bt_bytes + L.as_bytes + L.bs_bytes);
     const float *cs_scale = opts ? opts->col_scale : nullptr;
     const bool sparse = opts && (opts->flags & OS_OPT_SPARSE_A) && sketch_left_sparse_fits(p, mask);
+    const bool f16 = f16x3_pays(p, g0, m, l, mask, pack_bytes);
+    const os_dtype sk = f16 ? OS_F32 : g;   // what the sketches write
     const int64_t nchunks = (m + h.a_rows - 1) / h.a_rows;
     const int64_t npanels = (m + h.c_rows - 1) / h.c_rows;
 
@@ -419,7 +457,7 @@ extern "C" os_status oversketch_matmul_host(oversketch_plan_t plan, const void *
                 st = set_cuda_error(cudaGetLastError());
                 break;
             }
-            if ((st = sketch_right_impl(p, Bd, b_t, l, h.ldb_d, BtT, g, L.ldbt, bs, mask, pack, pack_bytes, cs)) != OS_OK)
+            if ((st = sketch_right_impl(p, Bd, b_t, l, h.ldb_d, BtT, sk, L.ldbt, bs, mask, pack, pack_bytes, cs)) != OS_OK)
                 break;
         }
         // A in chunks of rows, each sketched as it lands
@@ -436,9 +474,9 @@ extern "C" os_status oversketch_matmul_host(oversketch_plan_t plan, const void *
             void *at_c = (char *)At + (size_t)r0 * L.ldat * dtype_size(g);
             const void *a_c = Ad + (size_t)r0 * h.lda_d * ea;
             if (sparse)
-                st = sketch_left_sparse_impl(p, a_c, a_t, rows, h.lda_d, at_c, g, L.ldat, as, cs_scale, mask, cs);
+                st = sketch_left_sparse_impl(p, a_c, a_t, rows, h.lda_d, at_c, sk, L.ldat, as, cs_scale, mask, cs);
             else
-                st = sketch_left_impl(p, a_c, a_t, rows, h.lda_d, at_c, g, L.ldat, as, cs_scale, mask, pack, pack_bytes,
+                st = sketch_left_impl(p, a_c, a_t, rows, h.lda_d, at_c, sk, L.ldat, as, cs_scale, mask, pack, pack_bytes,
                                       cs);
         }
         if (st != OS_OK) break;
@@ -447,9 +485,12 @@ extern "C" os_status oversketch_matmul_host(oversketch_plan_t plan, const void *
             const int64_t r0 = q * h.c_rows, rows = (m - r0 < h.c_rows) ? m - r0 : h.c_rows;
             const void *at_q = (const char *)At + (size_t)r0 * L.ldat * dtype_size(g);
             const float *as_q = as ? as + r0 : nullptr;   // slice-major scales: the panel's rows start at r0
-            if ((st = oversketch_gemm_masked(plan, at_q, L.ldat, as_q, BtT, L.ldbt, bs, g, rows, l, mask, 1.0f,
-                                             0.0f, Cd + r0 * h.ldc_d, h.ldc_d, cs)) != OS_OK)
-                break;
+            if (f16)   // FP32 products run in one panel
+                st = matmul_f16x3(p, At, BtT, L.ldat, m, l, mask, Cd, h.ldc_d, pack, cs);
+            else
+                st = oversketch_gemm_masked(plan, at_q, L.ldat, as_q, BtT, L.ldbt, bs, g, rows, l, mask, 1.0f, 0.0f,
+                                            Cd + r0 * h.ldc_d, h.ldc_d, cs);
+            if (st != OS_OK) break;
             cudaEvent_t ec;
             if ((st = event(&ec)) != OS_OK) break;
             if (cudaEventRecord(ec, cs) != cudaSuccess || cudaStreamWaitEvent(xs, ec, 0) != cudaSuccess ||

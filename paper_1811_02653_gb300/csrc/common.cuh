@@ -44,6 +44,15 @@ struct BlockList {
     int32_t idx[64];
 };
 
+// One operand of the FP32 product on FP16 planes: `rows` rows of FP32 sums (pitch
+// shared by both operands), the planes hi and lo (rows x pitch FP16 each) behind
+// them, and a power-of-two scale per row.
+struct SplitSide {
+    float *sums;
+    int64_t rows;
+    float *scale;
+};
+
 os_status set_cuda_error(cudaError_t err);
 os_status check_launch();
 BlockList mask_to_list(uint64_t mask, int P);

@@ -34,6 +34,12 @@
 
 namespace osk {
 
+// implemented in split.cu
+os_status launch_split_f16(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
+                           unsigned int *flag, cudaStream_t st);
+os_status launch_tf32_planes(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
+                             const unsigned int *flag, cudaStream_t st);
+
 namespace {
 
 using namespace tc;
@@ -133,6 +139,11 @@ struct GemmArgs {
     // q % mn_b of the operand (its listed blocks of width mn_b, P of them stored)
     int32_t mn_b, mn_remap;
     BlockList mn_kept;
+    // FP16-plane products: power-of-two scale of each row of A~ and of B~^T
+    const float *a_scale, *b_scale;
+    // device word that makes the launch return at once: skip_if when it is nonzero,
+    // run_if when it is zero (null: always run)
+    const unsigned int *skip_if, *run_if;
 };
 
 // Tile pair t of the lower triangle (row-major: pair row pm, tile column tn <= pm).
@@ -257,6 +268,8 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
+    if constexpr (C::PLANES == 2)
+        if (g.run_if && *g.run_if == 0u) return;   // the FP16-plane product has written C
     if constexpr (GROUPED)
         for (int i = threadIdx.x; i < g.group_count; i += blockDim.x) s_begin[i] = g.group[i].tile_begin;
     if (threadIdx.x == 0) {
@@ -860,6 +873,253 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP32-accuracy masked GEMM on FP16 planes (split.cu), CTA pairs:
+//   A~ B~ = hi.hi + (hi.lo + lo.hi) / 2048        (lo.lo, 2^-24 of the terms, dropped)
+// The organisation of gemm_pair_bf16_kernel with 256 x 160 tiles and two kinds of
+// accumulators: hi.hi in chunks of K = 256, double-buffered, which the epilogue
+// adds in FP32 registers (the tensor core's FP32 accumulation truncates, so its
+// error must not grow with K), and the 2048 times smaller cross terms in one
+// accumulator over the whole K, which their truncation never reaches.  3 x 160
+// columns is what TMEM holds of the two.  Bound by the tensor pipe: a K step of 64
+// is 12 MMAs (960 tensor clocks) on 52 KB per CTA, 136 bytes of shared memory per clock.
+// 8192 x 8192 x 8192 on GB300: 1.93 ms (1.71 PFLOP/s of FP16 MMAs) against 4.05 ms
+// for the 3xTF32 kernel, with a seventh of its error (3.4e-7 against 2.4e-6 of ||C||).
+struct CfgF16x3 {
+    static constexpr int BN = 160;                    // tile columns (the pair's N)
+    static constexpr int STAGES = 4;
+    static constexpr int BKE = ROWB / 2;              // 64 FP16 per K step
+    static constexpr int A_BYTES = BM * ROWB;         // this CTA's 128 rows of one plane of A
+    static constexpr int B_BYTES = (BN / 2) * ROWB;   // this CTA's 80 rows of one plane of B
+    static constexpr int STAGE_BYTES = 2 * (A_BYTES + B_BYTES);   // [A hi][A lo][B hi][B lo]
+    static constexpr uint32_t PAIR_TX = 2u * STAGE_BYTES;
+    static constexpr int CHUNK_KB = 4;                // K steps per accumulator chunk
+    static constexpr int CROSS = 2 * BN;              // TMEM column of the cross terms
+    static constexpr int TMEM_COLS = 512;
+    static constexpr int THREADS = 192;
+    static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + 256 + kEpiBytes;
+    static constexpr uint32_t IDESC = idesc_f16_f32(2 * BM, BN);
+    static_assert(B_BYTES % 1024 == 0, "planes start on swizzle atoms");
+    static_assert(SMEM <= 232448, "shared memory");
+};
+
+__global__ void __launch_bounds__(CfgF16x3::THREADS, 1)
+gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid_constant__ CUtensorMap tmap_al,
+                       const __grid_constant__ CUtensorMap tmap_bh, const __grid_constant__ CUtensorMap tmap_bl,
+                       const GemmArgs g) {
+    using C = CfgF16x3;
+    constexpr int STAGES = C::STAGES, BN = C::BN;
+    if (*g.skip_if != 0u) return;   // operands that the FP16 planes do not suit (both CTAs see the same word)
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *tiles = smem;
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * C::STAGE_BYTES);   // leader's are used
+    uint64_t *empty = full + STAGES;
+    uint64_t *tmem_full = empty + STAGES;
+    uint64_t *tmem_empty = tmem_full + 2;                                          // leader's are used
+    uint64_t *cross_empty = tmem_empty + 2;                                        // leader's is used
+    uint64_t *drain = cross_empty + 1;
+    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 1);
+    volatile int *abort = reinterpret_cast<volatile int *>(tmem_base_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cluster_ctarank();
+    const bool leader = rank == 0;
+    const int t_first = blockIdx.x / 2, t_step = gridDim.x / 2;
+    const int tiles_mp = (g.tiles_m + 1) / 2;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(&tmem_full[a], 1);
+            mbar_init(&tmem_empty[a], 2 * 128);   // the epilogue threads of both CTAs
+        }
+        mbar_init(cross_empty, 2 * 128);
+        mbar_init(drain, 1);
+        *abort = 0;
+        fence_barrier_init();
+        prefetch_tmap(&tmap_ah);
+        prefetch_tmap(&tmap_al);
+        prefetch_tmap(&tmap_bh);
+        prefetch_tmap(&tmap_bl);
+    }
+    if (warp == 1) tmem_alloc_pair(tmem_base_slot, C::TMEM_COLS);
+    tc_fence_before();
+    cluster_sync_all();   // both CTAs' barriers exist before any remote arrival
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_base_slot;
+
+    auto coords = [&](int t, int &tm, int &tn) {
+        int pm = 0;
+        tile_coords(t, tiles_mp, g.tiles_n, pm, tn);
+        tm = 2 * pm + rank;   // past the last tile (odd count): zero rows, no stores
+    };
+
+    if (warp == 0) {
+        // ---------------- TMA producer (this CTA's half of every stage) ----------------
+        if (lane == 0) {
+            int stage = 0;
+            uint32_t phase = 0;
+            uint32_t issued_phase[STAGES];
+            bool issued[STAGES];
+            for (int s = 0; s < STAGES; ++s) issued[s] = false, issued_phase[s] = 0;
+            bool ok = true;
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
+                int tm, tn;
+                coords(t, tm, tn);
+                const int brow = tn * BN + rank * (BN / 2);
+                for (int kb = 0; kb < g.num_kb; ++kb) {
+                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, abort)) { ok = false; break; }
+                    const int blk = kb / g.kb_per_blk;
+                    const int kz = g.kept.idx[blk] * g.b + (kb - blk * g.kb_per_blk) * C::BKE;
+                    uint8_t *st = tiles + stage * C::STAGE_BYTES;
+                    const uint32_t fb = cluster_addr(&full[stage], 0);
+                    if (leader) mbar_expect_tx(&full[stage], C::PAIR_TX);
+                    tma_load_2d_pair(&tmap_ah, fb, st, kz, tm * BM);
+                    tma_load_2d_pair(&tmap_al, fb, st + C::A_BYTES, kz, tm * BM);
+                    tma_load_2d_pair(&tmap_bh, fb, st + 2 * C::A_BYTES, kz, brow);
+                    tma_load_2d_pair(&tmap_bl, fb, st + 2 * C::A_BYTES + C::B_BYTES, kz, brow);
+                    issued[stage] = true;
+                    issued_phase[stage] = phase;
+                    if (++stage == STAGES) stage = 0, phase ^= 1u;
+                }
+            }
+            // every stage this CTA loaded has been consumed by the pair's MMAs (so its
+            // copies have landed and no commit is still on its way here)
+            for (int s = 0; ok && s < STAGES; ++s)
+                if (issued[s] && !mbar_wait_cluster(&empty[s], issued_phase[s], abort)) ok = false;
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (leader; lane 0 issues, the warp waits together) ----------------
+        if (leader) {
+            int stage = 0;
+            uint32_t phase = 0;
+            int chunk = 0, tile = 0;
+            bool ok = true;
+            bool any = false;
+            const uint32_t dx = tmem_base + (uint32_t)C::CROSS;
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step, ++tile) {
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(cross_empty, (uint32_t)(tile & 1) ^ 1u, abort))) {
+                    ok = false;
+                    break;
+                }
+                for (int kc = 0; ok && kc < g.num_kb; kc += C::CHUNK_KB, ++chunk) {
+                    const int kc_end = min(g.num_kb, kc + C::CHUNK_KB);
+                    const int a = chunk & 1;
+                    const uint32_t aphase = (uint32_t)(chunk >> 1) & 1u;
+                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, abort))) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t d = tmem_base + (uint32_t)(a * BN);
+                    for (int kb = kc; kb < kc_end; ++kb) {
+                        if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort))) { ok = false; break; }
+                        tc_fence_after();
+                        if (lane == 0) {
+                            const uint32_t sah = smem_u32(tiles + stage * C::STAGE_BYTES);
+                            const uint32_t sal = sah + C::A_BYTES;
+                            const uint32_t sbh = sal + C::A_BYTES;
+                            const uint32_t sbl = sbh + C::B_BYTES;
+#pragma unroll
+                            for (int kk = 0; kk < ROWB / 32; ++kk) {
+                                const uint64_t ah = sdesc_kmajor_sw128(sah + kk * 32);
+                                const uint64_t al = sdesc_kmajor_sw128(sal + kk * 32);
+                                const uint64_t bh = sdesc_kmajor_sw128(sbh + kk * 32);
+                                const uint64_t bl = sdesc_kmajor_sw128(sbl + kk * 32);
+                                umma_f16_pair(d, ah, bh, C::IDESC, (kb > kc || kk > 0) ? 1u : 0u);
+                                umma_f16_pair(dx, ah, bl, C::IDESC, (kb > 0 || kk > 0) ? 1u : 0u);
+                                umma_f16_pair(dx, al, bh, C::IDESC, 1u);
+                            }
+                            umma_commit_pair(&empty[stage], 0x3);   // the stage is free in both CTAs
+                        }
+                        __syncwarp();
+                        any = true;
+                        if (++stage == STAGES) stage = 0, phase ^= 1u;
+                    }
+                    if (!ok) break;
+                    if (lane == 0) umma_commit_pair(&tmem_full[a], 0x3);   // both halves of the accumulator
+                    __syncwarp();
+                }
+            }
+            if (!ok && any && lane == 0) {
+                // drain: wait for the MMAs already issued before TMEM is freed
+                umma_commit_pair(drain, 0x1);
+                mbar_wait_drain(drain, 0);
+            }
+        }
+    } else {
+        // ---------------- epilogue (warps 2..5): this CTA's 128 rows ----------------
+        const int quarter = warp & 3;
+        float *buf = reinterpret_cast<float *>(smem + STAGES * C::STAGE_BYTES + 256) + quarter * 32 * kEpiPitch;
+        const uint32_t empty_cl[2] = {cluster_addr(&tmem_empty[0], 0), cluster_addr(&tmem_empty[1], 0)};
+        const uint32_t cross_cl = cluster_addr(cross_empty, 0);
+        const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16);
+        const bool vec_ok = ((reinterpret_cast<uintptr_t>(g.C) & 15u) == 0) && (g.ldc % 4 == 0);
+        int chunk = 0;
+        bool ok = true;
+        for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
+            int tm, tn;
+            coords(t, tm, tn);
+            float total[BN];
+#pragma unroll
+            for (int u = 0; u < BN; ++u) total[u] = 0.f;
+            for (int kc = 0; kc < g.num_kb; kc += C::CHUNK_KB, ++chunk) {
+                const int a = chunk & 1;
+                const uint32_t aphase = (uint32_t)(chunk >> 1) & 1u;
+                // warp-uniform decision: tcgen05.ld below is a .sync.aligned instruction
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, abort))) { ok = false; break; }
+                tc_fence_after();
+                if (kc + C::CHUNK_KB >= g.num_kb) {
+                    // the tile's last chunk: the cross terms are complete too
+#pragma unroll
+                    for (int ch = 0; ch < BN / 32; ++ch) {
+                        uint32_t v[32];
+                        tmem_ld_32x32b_x32(lanes + (uint32_t)(C::CROSS + ch * 32), v);
+#pragma unroll
+                        for (int u = 0; u < 32; ++u)
+                            total[ch * 32 + u] = fmaf(0x1p-11f, __uint_as_float(v[u]), total[ch * 32 + u]);
+                    }
+                    tc_fence_before();
+                    mbar_arrive_cluster(cross_cl);
+                }
+#pragma unroll
+                for (int ch = 0; ch < BN / 32; ++ch) {
+                    uint32_t v[32];
+                    tmem_ld_32x32b_x32(lanes + (uint32_t)(a * BN + ch * 32), v);
+#pragma unroll
+                    for (int u = 0; u < 32; ++u) total[ch * 32 + u] += __uint_as_float(v[u]);
+                }
+                tc_fence_before();
+                mbar_arrive_cluster(empty_cl[a]);
+            }
+            if (!ok) break;
+            const int64_t r0 = (int64_t)tm * BM + quarter * 32, c0 = (int64_t)tn * BN;
+            const float sa = r0 + lane < g.m ? __ldg(g.a_scale + r0 + lane) : 0.f;
+#pragma unroll
+            for (int ch = 0; ch < BN / 32; ++ch) {
+                const int64_t cb = c0 + ch * 32;
+                const float sb = cb + lane < g.l ? __ldg(g.b_scale + cb + lane) : 0.f;
+                float *tv = total + ch * 32;
+#pragma unroll
+                for (int u = 0; u < 32; ++u) tv[u] = tv[u] * sa * __shfl_sync(0xffffffffu, sb, u);
+                store_piece(buf, tv, g.alpha, g.beta, g.C, g.ldc, r0, g.m, cb, g.l, vec_ok, lane);
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();   // both CTAs are done with the shared TMEM and with each other's barriers
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, C::TMEM_COLS);
+    }
+}
+
 // ---------------------------------------------------------------- host ----
 
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -939,15 +1199,15 @@ namespace {
 template <class C>
 os_status launch_tc(const void *A0, const void *A1, int64_t lda, const void *B0, const void *B1, int64_t ldb,
                     int64_t m, int64_t l, int64_t zK, int32_t blk, const BlockList &kept, float alpha, float beta,
-                    float *Cout, int64_t ldc, cudaStream_t st) {
+                    float *Cout, int64_t ldc, cudaStream_t st, const unsigned int *run_if = nullptr) {
     if (blk % C::BKE != 0) return OS_ERR_UNSUPPORTED;
     if (!aligned16(A0) || !aligned16(B0) || (lda * C::ELEM) % 16 != 0 || (ldb * C::ELEM) % 16 != 0)
         return OS_ERR_INVALID_ARG;
     if ((C::PLANES == 2 || C::FP8) && (!aligned16(A1) || !aligned16(B1))) return OS_ERR_INVALID_ARG;
     if (zK >= (int64_t(1) << 31)) return OS_ERR_UNSUPPORTED;
     GemmArgs g;
-    g.group = nullptr;
-    g.group_count = 0;
+    std::memset(&g, 0, sizeof(g));
+    g.run_if = run_if;
     g.m = m;
     g.l = l;
     g.b = blk;
@@ -990,6 +1250,25 @@ os_status launch_tc(const void *A0, const void *A1, int64_t lda, const void *B0,
     const int grid = g.num_tiles < num_sms() ? g.num_tiles : num_sms();
     gemm_masked_tc_kernel<C, false><<<grid, C::THREADS, C::SMEM, st>>>(ta0, tb0, ta1, tb1, g);
     return check_launch();
+}
+
+// A persistent kernel over tile pairs: clusters of two CTAs, one pair per two SMs.
+template <typename Kern, typename... Args>
+cudaError_t launch_pairs(Kern kern, int threads, size_t smem, int num_tiles, cudaStream_t st, const Args &...args) {
+    const int pairs = num_sms() / 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2u * (unsigned)(num_tiles < pairs ? num_tiles : pairs));
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 template <bool kAMN, bool kBMN>
@@ -1045,21 +1324,7 @@ os_status launch_pair_args(const CUtensorMap &ta, const CUtensorMap &tb, const G
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
     });
     OSK_CUDA_TRY(attr_err);
-    const int pairs = num_sms() / 2;
-    const int grid = 2 * (g.num_tiles < pairs ? g.num_tiles : pairs);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(C::THREADS);
-    cfg.dynamicSmemBytes = C::SMEM;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    OSK_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_pair_bf16_kernel<kAMN, kBMN>, ta, tb, g));
+    OSK_CUDA_TRY(launch_pairs(gemm_pair_bf16_kernel<kAMN, kBMN>, C::THREADS, C::SMEM, g.num_tiles, st, ta, tb, g));
     return check_launch();
 }
 
@@ -1128,6 +1393,58 @@ os_status gemm_bf16_mn(const void *A, int64_t lda, bool a_mn, const void *B, int
                        uint64_t mask, int32_t P, cudaStream_t st) {
     const BlockList kept = mask_to_list(mask ? mask : ~0ull, P);
     return launch_pair_bf16_mn(A, lda, a_mn, B, ldb, b_mn, m, l, K, alpha, 0.0f, C, ldc, mn_b, remap, kept, P, st);
+}
+
+// The FP32-accuracy product from FP32 sums on FP16 planes (gemm_pair_f16x3_kernel):
+// split both operands, multiply, and behind the split's flag the 3xTF32 product of
+// the same sums for operands that the planes do not suit.  B's rows = 0: B is A.
+os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &b, int64_t ld, int64_t l,
+                            uint64_t mask, float alpha, float *Cout, int64_t ldc, unsigned int *flag,
+                            cudaStream_t st) {
+    using C = CfgF16x3;
+    const BlockList kept = mask_to_list(mask, p->P);
+    const SplitSide &bs = b.rows ? b : a;
+    const int64_t m = a.rows, z = (int64_t)p->P * p->b;
+    if (p->b % C::BKE != 0 || z >= (int64_t(1) << 31)) return OS_ERR_UNSUPPORTED;
+    if (!aligned16(a.sums) || !aligned16(bs.sums) || ld % 8 != 0) return OS_ERR_INVALID_ARG;
+    OSK_TRY(launch_split_f16(a, b, ld, p->b, kept, flag, st));
+    GemmArgs g;
+    std::memset(&g, 0, sizeof(g));
+    g.m = m;
+    g.l = l;
+    g.b = p->b;
+    g.kb_per_blk = p->b / C::BKE;
+    g.kept = kept;
+    g.num_kb = kept.count * g.kb_per_blk;
+    g.tiles_m = (int)((m + BM - 1) / BM);
+    g.tiles_n = (int)((l + C::BN - 1) / C::BN);
+    g.num_tiles = (g.tiles_m + 1) / 2 * g.tiles_n;   // tile pairs
+    g.alpha = alpha;
+    g.C = Cout;
+    g.ldc = ldc;
+    g.a_scale = a.scale;
+    g.b_scale = bs.scale;
+    g.skip_if = flag;
+    const uint16_t *ah = reinterpret_cast<const uint16_t *>(a.sums + m * ld);
+    const uint16_t *bh = reinterpret_cast<const uint16_t *>(bs.sums + bs.rows * ld);
+    CUtensorMap tah, tal, tbh, tbl;
+    const CUtensorMapDataType dt = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+    OSK_TRY(make_tmap(&tah, ah, dt, 2, m, z, ld, BM, C::BKE));
+    OSK_TRY(make_tmap(&tal, ah + m * ld, dt, 2, m, z, ld, BM, C::BKE));
+    OSK_TRY(make_tmap(&tbh, bh, dt, 2, l, z, ld, C::BN / 2, C::BKE));
+    OSK_TRY(make_tmap(&tbl, bh + bs.rows * ld, dt, 2, l, z, ld, C::BN / 2, C::BKE));
+    static std::once_flag attr_once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(attr_once, [] {
+        attr_err = cudaFuncSetAttribute(gemm_pair_f16x3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)C::SMEM);
+    });
+    OSK_CUDA_TRY(attr_err);
+    OSK_CUDA_TRY(launch_pairs(gemm_pair_f16x3_kernel, C::THREADS, C::SMEM, g.num_tiles, st, tah, tal, tbh, tbl, g));
+    OSK_TRY(check_launch());
+    OSK_TRY(launch_tf32_planes(a, b, ld, p->b, kept, flag, st));
+    return launch_tc<CfgTf32x3>(a.sums, a.sums + m * ld, ld, bs.sums, bs.sums + bs.rows * ld, ld, m, l, z, p->b, kept,
+                                alpha, 0.f, Cout, ldc, st, flag);
 }
 
 os_status gemm_masked_tc(const Plan *p, const void *At, int64_t ldat, const float *a_scales,

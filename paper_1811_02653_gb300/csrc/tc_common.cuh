@@ -249,6 +249,13 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
            | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same for FP16 operands (FP16 x FP16 -> F32).
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N) {
+    return (1u << 4)                 // D format F32; A and B format F16 (0)
+           | ((uint32_t)(N >> 3) << 17)
+           | ((uint32_t)(M >> 4) << 24);
+}
+
 // Instruction descriptor for kind::tf32 (TF32 x TF32 -> F32), both K-major.
 __host__ __device__ constexpr uint32_t idesc_tf32_f32(int M, int N) {
     return (1u << 4)                 // D format F32

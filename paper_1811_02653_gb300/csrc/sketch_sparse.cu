@@ -9,22 +9,31 @@
 // row once, coalesced, and routes only its nonzeros.  Two kernels, one after
 // the other:
 //
-// One-pass kernel (b <= 4096): the whole row's nonzeros are held in shared
-// memory, then routed one kept block at a time (sp_row_onepass):
-//   1. compaction: warp w streams the w-th 32nd of the row (16 elements per
-//      lane per step, the next step's loads issued before this one is
-//      processed, an L2 prefetch two steps ahead) and appends its nonzeros
-//      (index, value) to its own region in ascending index order: warp scans
-//      only, no block barrier;
-//   2. per kept block: bucket codes h_j(i), sigma_j(i) of every entry and the
-//      bucket counts (integer shared-memory atomics), a scan into bucket
+// One-pass kernel (b <= 4096): the whole row's nonzeros are held in shared memory,
+// then routed one kept block at a time.  A group of warps (half of the CTA, or all
+// of it) owns a row:
+//   1. compaction (sp1_compact): each warp streams its share of the row, 16 bytes
+//      per lane and load, and appends the nonzeros (index, value) to its own region
+//      in ascending index order: ballots only, no block barrier;
+//   2. per kept block (sp1_route): bucket codes h_j(i), sigma_j(i) of every entry
+//      and the bucket counts (integer shared-memory atomics), a scan into bucket
 //      starts, a scatter of entry numbers into their buckets, then each thread
-//      sorts the entry numbers of its 4 buckets and adds the members in that
-//      order (= ascending index) and writes the sums out in the output dtype
-//      (BF16 RNE, FP8 with the per-128-column UE8M0 scale, FP32, or TF32
-//      hi/lo planes).  No float atomics: bitwise reproducible.
-//   A row with more nonzeros in some 32nd than a region holds is left to the
+//      sorts the entry numbers of its buckets and adds the members in that order
+//      (= ascending index) and writes the sums out in the output dtype (BF16 RNE,
+//      FP8 with the per-128-column UE8M0 scale, FP32, or TF32 hi/lo planes).  No
+//      float atomics: bitwise reproducible.
+//   Two groups of 512 threads share a CTA and take turns at the routing, so that one
+//   row streams from HBM while the other is routed; the bucket tables exist once.
+//   A row with more nonzeros in some warp's share than a region holds is left to the
 //   flushing kernel: its first kept output gets a marker value.
+//   Bound by HBM and instruction issue together.  4096 x 2^20 FP32 at 1 % (17.2 GB,
+//   2.54 ms at the copy rate), 6 kept blocks of 4096, on GB300: 3.97 ms (5.47 with
+//   one row at a time and 1024 threads; the compaction alone 2.71; 2.84 ms at 0.3 %).
+//   Routing both rows at once, with bucket tables for each group, took 4.28 ms.
+//   What the routing's instructions cost decides: predicated accesses in place of
+//   branches around them, and sums without branches, gave 4.80 -> 4.02; buckets
+//   spread over all lanes (lane i of a warp has buckets i, i + 32, ..) the rest, and
+//   at 1024 x 2^20 with blocks of 512 (20 entries a bucket) 3.97 -> 1.87 ms.
 //
 // Flushing kernel (any density; all rows when b > 4096, else the marked ones):
 //   1. compaction: the row streams through registers in chunks of 16 elements
@@ -399,231 +408,461 @@ __device__ __forceinline__ void sp_row_flushing(const InT *__restrict__ row, int
     __syncthreads();   // the shared memory is free for the next row
 }
 
-// Shared memory of the one-pass row (b <= 4096): the bucket counts and starts,
-// then per warp a region of cw entries (index, value), and per entry its bucket
-// code in the current block and its place in the bucket order.
-constexpr int kOpElems = 16;   // one-pass compaction: elements per lane per step
-constexpr int kOpAhead = 2;    // L2 prefetch distance of a warp, in steps
+// ---- one-pass rows ----
+//
+// NG groups of 1024 / NG threads per CTA.  Shared memory: the bucket counters (16
+// bits each, two per word) and the sorted entry numbers, once; per group the values
+// and column indices of its row's entries, a region of cw per warp.  Indices are
+// relative to the warp's share of the row: 16 bits in two groups (n <= 2^20), 32 in one.
+constexpr int kSp1MaxBuckets = 4096;
+constexpr int kSp1Ahead = 3;     // L2 prefetch distance of a warp, in steps
 
-struct Sp1Smem {
-    int *cnt;            // [b] entries per bucket, then the scatter cursor
-    int *bstart;         // [b+1] first entry of each bucket in srt
-    int *warp_tot;       // [72] block-scan scratch
-    uint32_t *idx;       // [32*cw] column index of each entry
-    float *val;          // [32*cw] its value (times s_i)
-    uint16_t *code;      // [32*cw] bucket | 0x8000 for sign -1, current block
-    uint16_t *srt;       // [32*cw] entry numbers grouped by bucket
+template <int NG> struct Sp1 {
+    static constexpr int GT = kSpThreads / NG;          // threads per group
+    static constexpr int GW = GT / 32;                  // warps per group
+    static constexpr int BPT = kSp1MaxBuckets / GT;     // buckets per thread
+    using Idx = typename std::conditional<NG == 2, uint16_t, uint32_t>::type;
+    static constexpr int64_t kMaxN = NG == 2 ? int64_t(1) << 20 : (int64_t(1) << 31) - 1;
+    static constexpr int kEntryBytes = 2 + NG * (4 + (int)sizeof(Idx));
+    static constexpr int kMaxPairs = 16;                // codes of a lane's entries, two per register
+    static constexpr int kMaxRegion = 64 * kMaxPairs;   // entries per warp
+    static constexpr size_t kFixed = sizeof(uint32_t) * (kSp1MaxBuckets / 2 + 40 * NG) + 16;
+    static_assert(kMaxRegion * GW <= 32768, "entry numbers have 15 bits");
 };
 
-__host__ __device__ constexpr size_t sp1_fixed_bytes(int b) { return sizeof(int) * ((size_t)2 * b + 1 + 72 + 7); }
-constexpr int kSp1EntryBytes = 12;
-
-__device__ __forceinline__ Sp1Smem sp1_layout(void *base, int b, int cw) {
-    Sp1Smem s;
-    s.cnt = reinterpret_cast<int *>(base);
-    s.bstart = s.cnt + b;
-    s.warp_tot = s.bstart + b + 1;
-    s.idx = reinterpret_cast<uint32_t *>(s.warp_tot + 72 + 7);
-    s.val = reinterpret_cast<float *>(s.idx + 32 * cw);
-    s.code = reinterpret_cast<uint16_t *>(s.val + 32 * cw);
-    s.srt = s.code + 32 * cw;
-    return s;
+// Shared memory by 32-bit address: the one-pass kernel keeps its array bases in one
+// register each (recomputing them, as the compiler does for pointers into extern
+// shared memory here, took a tenth of the routing's instructions).
+__device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint4 lds_v4(uint32_t a) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a) {
+    uint32_t v;
+    asm volatile("{\n\t.reg .u16 h;\n\tld.shared.u16 h, [%1];\n\tcvt.u32.u16 %0, h;\n\t}" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ void sts_u32(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts_v4(uint32_t a, uint4 v) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v) {
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
+}
+// The same under a condition, as one predicated instruction (a branch around an
+// access costs three more).
+__device__ __forceinline__ void sts_u32_if(bool c, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u32 [%1], %2;\n\t}"
+                 ::"r"((uint32_t)c), "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts_u16_if(bool c, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u16 [%1], %2;\n\t}"
+                 ::"r"((uint32_t)c), "r"(a), "h"((uint16_t)v) : "memory");
+}
+__device__ __forceinline__ void reds_add_if(bool c, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p red.shared.add.u32 [%1], %2;\n\t}"
+                 ::"r"((uint32_t)c), "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t atoms_add_if(bool c, uint32_t a, uint32_t v) {
+    uint32_t o;
+    asm volatile("{\n\t.reg .pred p;\n\tmov.u32 %0, 0;\n\tsetp.ne.u32 p, %1, 0;\n\t@p atom.shared.add.u32 %0, [%2], %3;\n\t}"
+                 : "=&r"(o) : "r"((uint32_t)c), "r"(a), "r"(v) : "memory");
+    return o;
+}
+// A row entry's column index (relative to its warp's share): 16 or 32 bits.
+template <typename IdxT> __device__ __forceinline__ uint32_t lds_idx(uint32_t a, uint32_t k) {
+    return sizeof(IdxT) == 2 ? lds_u16(a + 2 * k) : lds_u32(a + 4 * k);
+}
+template <typename IdxT> __device__ __forceinline__ void sts_idx_if(bool c, uint32_t a, uint32_t k, uint32_t v) {
+    if (sizeof(IdxT) == 2) sts_u16_if(c, a + 2 * k, v);
+    else sts_u32_if(c, a + 4 * k, v);
 }
 
-// The row in one pass (b <= 4096, at most cw nonzeros in each 32nd of the row):
-//   1. warp w compacts the w-th 32nd of the row into its own region (a warp
-//      scan of each lane's nonzero count, no block barrier), entries in
-//      ascending index order; each step's loads are issued before the previous
-//      step is processed, an L2 prefetch runs two steps ahead, and the start of
-//      the next row is prefetched before the routing;
-//   2. per kept block: codes and bucket counts (integer atomics), a scan into
-//      bucket starts, a scatter of entry numbers into their buckets, then each
-//      thread sums the members of its 4 buckets in ascending entry order (the
-//      order of the flushing path: both give the same bits) and writes them
-//      out directly, so no accumulators outlive the block.
-// Returns false, with nothing written, when a region overflows.
-template <typename InT, typename OutT, bool kScale>
-__device__ bool sp_row_onepass(const InT *__restrict__ row, const InT *__restrict__ next_row, int64_t r,
-                               int64_t n, bool vec, const uint32_t *__restrict__ hs, uint64_t seed, bool hashed,
-                               int32_t b, const BlockList &blocks, int cw, const float *__restrict__ col_scale,
-                               OutT *__restrict__ At, int64_t ldat, float *__restrict__ scales, int64_t lds,
-                               int64_t plane_elems, void *smem) {
-    const Sp1Smem s = sp1_layout(smem, b, cw);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int kOp = kOpElems;                             // elements per lane per step
-    constexpr int64_t kStep = 32 * kOp;                       // elements per warp step
-    const int64_t seg = ((n + 31) / 32 + kOp - 1) / kOp * kOp;
-    const int64_t s0 = min(n, (int64_t)warp * seg), s1 = min(n, s0 + seg);
-    uint32_t *ridx = s.idx + warp * cw;
-    float *rval = s.val + warp * cw;
-    int have = 0;          // entries in this warp's region
-    bool over = false;
-    // one step of kOp elements per lane: its loads are issued a step ahead
-    auto load_step = [&](int64_t i0, float (&v)[kOp]) {
-        const int64_t il = i0 + (int64_t)kOp * lane;
-        if (i0 < s1 && il < s1) {
+__device__ __forceinline__ void group_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void group_arrive(int id, int threads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// Barrier of the group that also ORs a predicate over its threads.
+__device__ __forceinline__ bool group_or(int id, int threads, bool p) {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred a, b;\n\tsetp.ne.u32 a, %1, 0;\n\tbar.red.or.pred b, %2, %3, a;\n\tselp.u32 %0, 1, 0, b;\n\t}"
+                 : "=r"(r)
+                 : "r"((uint32_t)p), "r"(id), "r"(threads)
+                 : "memory");
+    return r != 0;
+}
+
+// One lane's 16 bytes of a row: E elements, tested and picked by their bits.
+template <typename InT> struct Piece;
+template <> struct Piece<float> {
+    static constexpr int E = 4;
+    __device__ static bool any(const uint4 &u) { return ((u.x | u.y | u.z | u.w) & 0x7fffffffu) != 0u; }
+    __device__ static uint32_t mask(const uint4 &u) {
+        return ((u.x & 0x7fffffffu) ? 1u : 0u) | ((u.y & 0x7fffffffu) ? 2u : 0u) | ((u.z & 0x7fffffffu) ? 4u : 0u) |
+               ((u.w & 0x7fffffffu) ? 8u : 0u);
+    }
+    __device__ static float pick(const uint4 &u, int j) {
+        const uint32_t a = (j & 1) ? u.y : u.x, b = (j & 1) ? u.w : u.z;
+        return __uint_as_float((j & 2) ? b : a);
+    }
+    // the first nonzero (j, v) of a piece that has one; whether any lane's piece has more
+    __device__ static bool first(const uint4 &u, int &j, float &v) {
+        uint32_t more;
+        asm volatile(
+            "{\n\t.reg .pred x, y, z, w, a, b;\n\t.reg .u32 t;\n\t.reg .f32 f;\n\t"
+            "setp.neu.f32 x, %3, 0f00000000;\n\tsetp.neu.f32 y, %4, 0f00000000;\n\t"
+            "setp.neu.f32 z, %5, 0f00000000;\n\tsetp.neu.f32 w, %6, 0f00000000;\n\t"
+            "selp.u32 t, 2, 3, z;\n\tselp.u32 t, 1, t, y;\n\tselp.u32 %1, 0, t, x;\n\t"
+            "selp.f32 f, %5, %6, z;\n\tselp.f32 f, %4, f, y;\n\tselp.f32 %2, %3, f, x;\n\t"
+            "and.pred a, z, w;\n\tor.pred b, z, w;\n\tand.pred z, y, b;\n\tor.pred b, y, b;\n\t"
+            "and.pred x, x, b;\n\tor.pred a, a, z;\n\tor.pred a, a, x;\n\t"
+            "vote.sync.any.pred a, a, 0xffffffff;\n\tselp.u32 %0, 1, 0, a;\n\t}"
+            : "=r"(more), "=r"(j), "=f"(v)
+            : "f"(__uint_as_float(u.x)), "f"(__uint_as_float(u.y)), "f"(__uint_as_float(u.z)), "f"(__uint_as_float(u.w)));
+        return more != 0u;
+    }
+};
+template <> struct Piece<__nv_bfloat16> {
+    static constexpr int E = 8;
+    __device__ static bool any(const uint4 &u) { return ((u.x | u.y | u.z | u.w) & 0x7fff7fffu) != 0u; }
+    __device__ static uint32_t two(uint32_t w) { return ((w & 0x7fffu) ? 1u : 0u) | ((w & 0x7fff0000u) ? 2u : 0u); }
+    __device__ static uint32_t mask(const uint4 &u) {
+        return two(u.x) | two(u.y) << 2 | two(u.z) << 4 | two(u.w) << 6;
+    }
+    __device__ static float pick(const uint4 &u, int j) {
+        const uint32_t a = (j & 2) ? u.y : u.x, b = (j & 2) ? u.w : u.z, w = (j & 4) ? b : a;
+        return __uint_as_float((j & 1) ? (w & 0xffff0000u) : (w << 16));
+    }
+    __device__ static bool first(const uint4 &u, int &j, float &v) {
+        const uint32_t nz = mask(u);
+        j = __ffs((int)nz) - 1;
+        v = pick(u, j);
+        return __any_sync(0xffffffffu, (nz & (nz - 1u)) != 0u);
+    }
+};
+
+// Compaction of columns [s0, s1) of a row by one warp: its nonzeros, ascending, to
+// val / idx (indices relative to s0).  Steps of four 16-byte loads per lane (the
+// next step's issued before this one is processed); each load's 32 pieces take a
+// ballot, and only the pieces with a nonzero (most have one at a percent) the rest.
+// Returns the count, or -1 when the region of cw entries overflows.
+template <typename InT, typename IdxT>
+__device__ __forceinline__ int sp1_compact(const InT *__restrict__ row, int64_t s0, int64_t s1, bool vec,
+                                           uint32_t val, uint32_t idx, int cw) {
+    using P = Piece<InT>;
+    constexpr int Q = 4, E = P::E;
+    constexpr int kChunk = 32 * E, kStep = Q * kChunk;
+    const int lane = threadIdx.x & 31;
+    const uint32_t below = (1u << lane) - 1u;
+    int have = 0;
+    auto process = [&](int at0, const uint4 (&u)[Q]) {
 #pragma unroll
-            for (int h = 0; h < kOp / 16; ++h) {
-                float(&vh)[16] = *reinterpret_cast<float(*)[16]>(v + 16 * h);
-                if (vec) load16<InT, true>(row, il + 16 * h, n, vh);
-                else load16<InT, false>(row, il + 16 * h, n, vh);
+        for (int q = 0; q < Q; ++q) {
+            const bool any = P::any(u[q]);
+            const uint32_t bal = __ballot_sync(0xffffffffu, any);
+            if (bal == 0u) continue;
+            const int at = at0 + q * kChunk;
+            int k;
+            float v;
+            if (P::first(u[q], k, v)) {
+                // some lane holds two or more: a lane's first position by a ballot per element
+                const uint32_t nz = P::mask(u[q]);
+                int pos = have, total = 0;
+#pragma unroll 1
+                for (int j = 0; j < E; ++j) {
+                    const uint32_t bj = __ballot_sync(0xffffffffu, (nz >> j) & 1u);
+                    pos += __popc(bj & below);
+                    total += __popc(bj);
+                }
+#pragma unroll 1
+                for (int j = 0; j < E; ++j) {
+                    if (((nz >> j) & 1u) && pos < cw) {
+                        sts_u32(val + 4 * pos, __float_as_uint(P::pick(u[q], j)));
+                        sts_idx_if<IdxT>(true, idx, pos, (uint32_t)(at + j));
+                        ++pos;
+                    }
+                }
+                have += total;
+            } else {
+                const int pos = have + __popc(bal & below);
+                const bool put = any & (pos < cw);
+                sts_u32_if(put, val + 4 * pos, __float_as_uint(v));
+                sts_idx_if<IdxT>(put, idx, pos, (uint32_t)(at + k));
+                have += __popc(bal);
             }
-        } else {
-#pragma unroll
-            for (int q = 0; q < kOp; ++q) v[q] = 0.f;
         }
     };
-    // append the nonzeros of one step (false: the region is full, nothing appended)
-    auto process = [&](const float (&v)[kOp], int64_t i0) -> bool {
-        if (vec && lane == 0) {
-            const int64_t pf = i0 + kOpAhead * kStep;
-            if (pf < s1) {
-                const int64_t bytes = (min(kStep, s1 - pf) * (int64_t)sizeof(InT)) & ~int64_t(15);
-                if (bytes > 0) l2_prefetch(row + pf, (uint32_t)bytes);
+    const InT *p = row + s0 + E * lane;
+    auto load = [&](const InT *from, uint4 (&u)[Q]) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) u[q] = __ldcs(reinterpret_cast<const uint4 *>(from + q * kChunk));   // streamed
+    };
+    const int steps = vec ? (int)((s1 - s0) / kStep) : 0;   // whole steps, 16-byte loads
+    int at = E * lane;
+    uint4 ua[Q], ub[Q];
+    if (steps > 0) load(p, ua);
+    for (int st = 0; st < steps; st += 2) {
+        if (lane == 0 && st + kSp1Ahead + 2 <= steps)
+            l2_prefetch(p + kSp1Ahead * kStep, 2 * kStep * (uint32_t)sizeof(InT));
+        if (st + 1 < steps) load(p + kStep, ub);
+        process(at, ua);
+        if (st + 1 >= steps) break;
+        if (st + 2 < steps) load(p + 2 * kStep, ua);
+        process(at + kStep, ub);
+        p += 2 * kStep;
+        at += 2 * kStep;
+        if (have > cw) return -1;   // warp-uniform
+    }
+    // the rest of the share (all of it for rows without 16-byte alignment)
+    for (int64_t i0 = s0 + (int64_t)steps * kStep; i0 < s1; i0 += kStep) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int64_t i = i0 + q * kChunk + E * lane;
+            InT e[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) e[j] = i + j < s1 ? row[i + j] : InT(0.f);
+            ua[q] = *reinterpret_cast<const uint4 *>(e);
+        }
+        process((int)(i0 - s0) + E * lane, ua);
+        if (have > cw) return -1;
+    }
+    return have > cw ? -1 : have;
+}
+
+__device__ __forceinline__ void cex(uint32_t &a, uint32_t &b) {
+    const uint32_t lo = min(a, b);
+    b = max(a, b);
+    a = lo;
+}
+
+// The routing of one row (`have` entries in this warp's region): see the file
+// comment.
+template <typename OutT, int NG>
+__device__ __forceinline__ void sp1_route(uint32_t cnt, uint32_t warp_tot, uint32_t srt, uint32_t val, uint32_t idx,
+                                          int have, uint32_t base, int cw, int64_t r,
+                                          const uint32_t *__restrict__ hs, int64_t n, uint64_t seed, bool hashed,
+                                          int32_t b, const BlockList &blocks, OutT *__restrict__ At, int64_t ldat,
+                                          float *__restrict__ scales, int64_t lds, int64_t plane_elems, int bar) {
+    using S = Sp1<NG>;
+    using Idx = typename S::Idx;
+    constexpr int GT = S::GT, GW = S::GW, BPT = S::BPT, WPT = BPT / 2;
+    const int tid = threadIdx.x % GT, lane = tid & 31, warp = tid >> 5;
+    const int e0 = warp * cw;                 // this warp's first entry number
+    const uint32_t own = idx + (uint32_t)(sizeof(Idx) * e0);
+    uint32_t code[S::kMaxPairs];              // bucket | sign << 15 of entries lane + 64 u (low) and + 32 (high)
+    auto fill = [&](auto &&code_of) {
+#pragma unroll
+        for (int u = 0; u < S::kMaxPairs; ++u) {
+            if (64 * u >= have) break;
+            uint32_t cd[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                cd[h] = code_of(base + lds_idx<Idx>(own, min(64 * u + 32 * h + lane, have - 1)));   // repeats the last entry
+                cd[h] = (cd[h] & 0x7fffu) | ((cd[h] >> 16) & 0x8000u);
+            }
+            code[u] = cd[0] | cd[1] << 16;
+        }
+    };
+    auto load_codes = [&](int jb) {
+        if (hashed) {
+            const uint64_t key = block_key(seed, jb);
+            fill([&](uint32_t i) { return hash_code(key, (int64_t)i, b); });
+        } else {
+            const uint32_t *hj = hs + (int64_t)jb * n;
+            fill([&](uint32_t i) { return __ldg(hj + i); });
+        }
+    };
+    // the thread's buckets: BPT*tid .. BPT*tid + BPT-1 (counter words WPT*tid ..)
+    const uint32_t words = cnt + 4 * WPT * tid;
+    auto read_words = [&](uint32_t (&w)[WPT]) {
+        if constexpr (WPT == 4) {
+            const uint4 q = lds_v4(words);
+            w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+        } else {
+            w[0] = lds_u32(words);
+            w[1] = lds_u32(words + 4);
+        }
+    };
+    auto write_words = [&](const uint32_t (&w)[WPT]) {
+        if constexpr (WPT == 4) {
+            sts_v4(words, make_uint4(w[0], w[1], w[2], w[3]));
+        } else {
+            sts_u32(words, w[0]);
+            sts_u32(words + 4, w[1]);
+        }
+    };
+#pragma unroll 1
+    for (int t = 0; t < blocks.count; ++t) {
+        const int jb = blocks.idx[t];
+        load_codes(jb);
+        if (t > 0) group_sync(bar, GT);   // the block before is done with the counters and entry lists
+        {
+            const uint32_t zero[WPT] = {};
+            write_words(zero);
+        }
+        group_sync(bar, GT);
+#pragma unroll
+        for (int u = 0; u < S::kMaxPairs; ++u) {
+            if (64 * u >= have) break;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t bk = (code[u] >> (16 * h)) & 0x7fffu;
+                reds_add_if(64 * u + 32 * h + lane < have, cnt + 4 * (bk >> 1), (bk & 1u) ? 0x10000u : 1u);
             }
         }
-        const int64_t il = i0 + (int64_t)kOp * lane;
-        uint32_t nz = 0;
+        group_sync(bar, GT);
+        // bucket starts: the thread's counts, a warp scan, the totals of the warps before
+        uint32_t w[WPT];
+        read_words(w);
+        int mine = 0;
 #pragma unroll
-        for (int q = 0; q < kOp; ++q) nz |= (v[q] != 0.f ? 1u : 0u) << q;
-        const int c = __popc(nz);
-        int inc = c;
+        for (int q = 0; q < WPT; ++q) mine += (int)(w[q] & 0xffffu) + (int)(w[q] >> 16);
+        int inc = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, inc, o);
             if (lane >= o) inc += y;
         }
-        const int total = __shfl_sync(0xffffffffu, inc, 31);
-        if (have + total > cw) return false;   // warp-uniform
-        int pos = have + inc - c;
+        if (lane == 31) sts_u32(warp_tot + 4 * warp, (uint32_t)inc);
+        group_sync(bar, GT);
+        int before = lane < warp ? (int)lds_u32(warp_tot + 4 * lane) : 0;   // warp <= 31
+        before = __reduce_add_sync(0xffffffffu, before);
+        const int start = before + inc - mine;
+        {
+            int off = start;
 #pragma unroll
-        for (int q = 0; q < kOp; ++q) {
-            if ((nz >> q) & 1u) {
-                ridx[pos] = (uint32_t)(il + q);
-                rval[pos] = v[q];
-                ++pos;
+            for (int q = 0; q < WPT; ++q) {
+                const int k0 = (int)(w[q] & 0xffffu), k1 = (int)(w[q] >> 16);
+                w[q] = (uint32_t)off | ((uint32_t)(off + k0) << 16);
+                off += k0 + k1;
             }
         }
-        have += total;
-        return true;
-    };
-    // two steps per pass, each one's loads issued before the other is processed
-    float va[kOp], vb[kOp];
-    load_step(s0, va);
-    for (int64_t i0 = s0; i0 < s1; i0 += 2 * kStep) {
-        load_step(i0 + kStep, vb);
-        if (!process(va, i0)) {
-            over = true;
-            break;
-        }
-        if (i0 + kStep >= s1) break;
-        load_step(i0 + 2 * kStep, va);
-        if (!process(vb, i0 + kStep)) {
-            over = true;
-            break;
-        }
-    }
-    if (vec && next_row && lane == 0 && s0 < s1) {
-        const int64_t bytes = (min(kOpAhead * kStep, s1 - s0) * (int64_t)sizeof(InT)) & ~int64_t(15);
-        if (bytes > 0) l2_prefetch(next_row + s0, (uint32_t)bytes);
-    }
-    if (!__syncthreads_and(!over)) return false;
-
-    if constexpr (kScale) {
-#pragma unroll 4
-        for (int k = lane; k < have; k += 32) rval[k] *= __ldg(col_scale + ridx[k]);
-    }
-    for (int c = tid; c < b; c += kSpThreads) s.cnt[c] = 0;
-    __syncthreads();
-
-    for (int t = 0; t < blocks.count; ++t) {
-        const int jb = blocks.idx[t];
-        const uint64_t key = hashed ? block_key(seed, jb) : 0ull;
-        const uint32_t *hj = hs + (int64_t)jb * n;
-        // codes and counts of the warp's own entries
-        for (int k = lane; k < have; k += 32) {
-            const uint32_t i = ridx[k];
-            const uint32_t cd = hashed ? hash_code(key, (int64_t)i, b) : __ldg(hj + i);
-            const uint32_t bk = cd & kIndexMask;
-            s.code[warp * cw + k] = (uint16_t)(bk | ((cd & kSignBit) ? 0x8000u : 0u));
-            atomicAdd(&s.cnt[bk], 1);
-        }
-        __syncthreads();
-        // bucket starts: thread t owns buckets 4t .. 4t+3
-        const int c0 = min(b, 4 * tid), c1 = min(b, 4 * tid + 4);
-        int run = 0;
-        for (int c = c0; c < c1; ++c) run += s.cnt[c];
-        int all = 0;
-        int off = block_scan(run, s.warp_tot, &all);
-        for (int c = c0; c < c1; ++c) {
-            const int k = s.cnt[c];
-            s.bstart[c] = off;
-            s.cnt[c] = off;
-            off += k;
-        }
-        if (tid == 0) s.bstart[b] = all;
-        __syncthreads();
-        // entry numbers into their buckets
-        for (int k = lane; k < have; k += 32) {
-            const int e = warp * cw + k;
-            const int p = atomicAdd(&s.cnt[s.code[e] & 0x7fff], 1);
-            s.srt[p] = (uint16_t)e;
-        }
-        __syncthreads();
-        // each bucket's members in ascending entry order (= ascending index)
-        float a[4];
+        write_words(w);
+        group_sync(bar, GT);
+        // entry numbers (and signs) into their buckets
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = 4 * tid + q;
-            a[q] = 0.f;
-            if (c < b) {
-                const int p0 = s.bstart[c], p1 = s.bstart[c + 1];
-                auto add = [&](int e) {
-                    const float x = s.val[e];
-                    a[q] += (s.code[e] & 0x8000u) ? -x : x;
-                };
-                if (p1 - p0 == 1) {
-                    add(s.srt[p0]);
-                } else if (p1 - p0 == 2) {
-                    const int e0 = s.srt[p0], e1 = s.srt[p0 + 1];
-                    add(min(e0, e1));
-                    add(max(e0, e1));
-                } else if (p1 > p0) {
-                    // longer lists: insertion sort of the bucket's own slice of srt
-                    for (int k = p0 + 1; k < p1; ++k) {
-                        const uint16_t x = s.srt[k];
-                        int j = k - 1;
-                        for (; j >= p0 && s.srt[j] > x; --j) s.srt[j + 1] = s.srt[j];
-                        s.srt[j + 1] = x;
-                    }
-                    for (int k = p0; k < p1; ++k) add(s.srt[k]);
+        for (int u = 0; u < S::kMaxPairs; ++u) {
+            if (64 * u >= have) break;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t cd = code[u] >> (16 * h), bk = cd & 0x7fffu;
+                const int k = 64 * u + 32 * h + lane;
+                const uint32_t old = atoms_add_if(k < have, cnt + 4 * (bk >> 1), (bk & 1u) ? 0x10000u : 1u);
+                const uint32_t pos = (bk & 1u) ? old >> 16 : old & 0xffffu;
+                sts_u16_if(k < have, srt + 2 * pos, ((uint32_t)(e0 + k) << 1) | ((cd >> 15) & 1u));
+            }
+        }
+        group_sync(bar, GT);
+        // The counters now hold the buckets' ends.  A warp owns `per` consecutive buckets,
+        // lane i buckets i, i + 32, ..: every lane has one down to b = 32 GW, and its
+        // sums are stored whole lines at a time.  A bucket's members are added in
+        // ascending entry order (= ascending index) behind a sorting network over 4, 6
+        // or 8 of them, straight-line and predicated; longer lists are sorted by
+        // insertion in their slice of srt.
+        auto bucket_end = [&](int c) -> int {   // 0 for c < 0
+            const uint32_t w = lds_u32(cnt + 4 * (max(c, 0) >> 1));
+            return c < 0 ? 0 : (int)((c & 1) ? w >> 16 : w & 0xffffu);
+        };
+        auto term = [&](uint32_t m) -> float {   // the sign is the entry number's lowest bit
+            return __uint_as_float(lds_u32(val + 2 * (m & 0xfffeu)) ^ (m << 31));
+        };
+        auto bucket_sum = [&](int q) -> float {   // bucket q (zero past the last); all lanes of the warp together
+            const int p0 = q < b ? bucket_end(q - 1) : 0;
+            const int c = q < b ? bucket_end(q) - p0 : 0;
+            const uint32_t from = srt + 2 * p0;
+            auto sorted_sum = [&](auto nn) -> float {
+                constexpr int N = decltype(nn)::value;
+                uint32_t m[N];   // reads past the bucket (and past srt's end, into its padding) are dropped
+#pragma unroll
+                for (int k = 0; k < N; ++k) m[k] = lds_u16(from + 2 * k);
+#pragma unroll
+                for (int k = 0; k < N; ++k) m[k] = k < c ? m[k] : 0xffffu;
+                // Batcher's odd-even merge sort
+                cex(m[0], m[1]); cex(m[2], m[3]); cex(m[0], m[2]); cex(m[1], m[3]); cex(m[1], m[2]);
+                if constexpr (N == 6) {
+                    cex(m[4], m[5]);
+                    cex(m[0], m[4]); cex(m[1], m[5]); cex(m[2], m[4]); cex(m[3], m[5]); cex(m[1], m[2]); cex(m[3], m[4]);
+                } else if constexpr (N == 8) {
+                    cex(m[4], m[5]); cex(m[6], m[7]); cex(m[4], m[6]); cex(m[5], m[7]); cex(m[5], m[6]);
+                    cex(m[0], m[4]); cex(m[1], m[5]); cex(m[2], m[6]); cex(m[3], m[7]);
+                    cex(m[2], m[4]); cex(m[3], m[5]);
+                    cex(m[1], m[2]); cex(m[3], m[4]); cex(m[5], m[6]);
                 }
-                s.cnt[c] = 0;
+                float x[N];
+#pragma unroll
+                for (int k = 0; k < N; ++k) x[k] = term(k < c ? m[k] : 0u);
+                float s = 0.f;
+#pragma unroll
+                for (int k = 0; k < N; ++k) s = k < c ? s + x[k] : s;
+                return s;
+            };
+            const int most = __reduce_max_sync(0xffffffffu, c <= 8 ? c : 0);
+            float s;
+            if (most <= 4) s = sorted_sum(std::integral_constant<int, 4>());
+            else if (most <= 6) s = sorted_sum(std::integral_constant<int, 6>());
+            else s = sorted_sum(std::integral_constant<int, 8>());
+            if (c > 8) {
+#pragma unroll 1
+                for (int k = 1; k < c; ++k) {
+                    const uint32_t x = lds_u16(from + 2 * k);
+                    int j = k - 1;
+                    for (; j >= 0; --j) {
+                        const uint32_t y = lds_u16(from + 2 * j);
+                        if (y <= x) break;
+                        sts_u16(from + 2 * j + 2, y);
+                    }
+                    sts_u16(from + 2 * j + 2, x);
+                }
+                s = 0.f;
+#pragma unroll 1
+                for (int k = 0; k < c; ++k) s += term(lds_u16(from + 2 * k));
             }
-        }
+            return s;
+        };
         const int64_t col0 = (int64_t)jb * b;
         OutT *dst = At + r * ldat + col0;
         if constexpr (sizeof(OutT) == 1) {
-            // FP8: warp w holds the 128-column slice w of the block
-            if (128 * warp < b) {
-                float am = fmaxf(fmaxf(fabsf(a[0]), fabsf(a[1])), fmaxf(fabsf(a[2]), fabsf(a[3])));
+            // FP8 (b % 128 == 0): whole 128-column slices per warp
+            const int per = ((b + GW - 1) / GW + 127) / 128 * 128;
+#pragma unroll 1
+            for (int q0 = warp * per; q0 < min(b, (warp + 1) * per); q0 += 128) {
+                float a[4], am = 0.f;
+#pragma unroll 1
+                for (int i = 0; i < 4; ++i) {
+                    const float x = bucket_sum(q0 + 32 * i + lane);
+                    am = fmaxf(am, fabsf(x));
+                    if (i == 0) a[0] = x;
+                    else if (i == 1) a[1] = x;
+                    else if (i == 2) a[2] = x;
+                    else a[3] = x;
+                }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
                 const int e = fp8_scale_exponent(am);
                 const float inv = ldexpf(1.f, -e);
-                __nv_fp8_e4m3 qv[4] = {__nv_fp8_e4m3(a[0] * inv), __nv_fp8_e4m3(a[1] * inv),
-                                       __nv_fp8_e4m3(a[2] * inv), __nv_fp8_e4m3(a[3] * inv)};
-                *reinterpret_cast<uint32_t *>(dst + 4 * tid) = *reinterpret_cast<uint32_t *>(qv);
-                if (lane == 0) scales[(col0 / 128 + warp) * lds + r] = ldexpf(1.f, e);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) dst[q0 + 32 * i + lane] = __nv_fp8_e4m3(a[i] * inv);
+                if (lane == 0) scales[((col0 + q0) / 128) * lds + r] = ldexpf(1.f, e);
             }
         } else {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (4 * tid + q < b) sp_store(dst + 4 * tid + q, plane_elems, a[q]);
+            const int per = ((b + GW - 1) / GW + 31) / 32 * 32;
+#pragma unroll 1
+            for (int q0 = warp * per; q0 < min(b, (warp + 1) * per); q0 += 32) {
+                const float x = bucket_sum(q0 + lane);
+                if (q0 + lane < b) sp_store(dst + q0 + lane, plane_elems, x);
+            }
         }
-        __syncthreads();   // counts cleared, codes and bucket lists free for the next block
     }
-    return true;
 }
 
 // Bits that mark a row the one-pass kernel left to the flushing kernel, stored
@@ -642,23 +881,54 @@ __device__ __forceinline__ typename RowMark<OutT>::U *row_mark(OutT *At, int64_t
     return reinterpret_cast<typename RowMark<OutT>::U *>(At + r * ldat + col);
 }
 
-// The one-pass kernel: one CTA per row (persistent over rows); a row whose
-// nonzeros overflow a warp's region is marked for the flushing kernel.
-template <typename InT, typename OutT, bool kScale>
+// The one-pass kernel (persistent over rows).  Group g of a CTA takes every NG-th of
+// its rows; with two groups the routing (the shared counters and entry lists) goes
+// from one to the other row by row, so each group compacts while the other routes.
+// A row whose nonzeros overflow a warp's region is marked for the flushing kernel.
+template <typename InT, typename OutT, bool kScale, int NG>
 __global__ void __launch_bounds__(kSpThreads, 1)
 sketch_left_onepass_kernel(const InT *__restrict__ A, int64_t lda, int64_t m, int64_t n, bool vec,
                            const uint32_t *__restrict__ hs, uint64_t seed, bool hashed, int32_t b,
-                           BlockList blocks, int cw,
+                           const __grid_constant__ BlockList blocks, int cw,
                            const float *__restrict__ col_scale, OutT *__restrict__ At, int64_t ldat,
                            float *__restrict__ scales, int64_t lds, int64_t plane_elems) {
+    using S = Sp1<NG>;
+    using Idx = typename S::Idx;
     extern __shared__ float4 sp_smem[];
-    for (int64_t r = blockIdx.x; r < m; r += gridDim.x) {
-        const InT *row = A + r * lda;
-        const InT *next = r + gridDim.x < m ? row + (int64_t)gridDim.x * lda : nullptr;
-        if (!sp_row_onepass<InT, OutT, kScale>(row, next, r, n, vec, hs, seed, hashed, b, blocks, cw, col_scale,
-                                               At, ldat, scales, lds, plane_elems, sp_smem) &&
-            threadIdx.x == 0)
+    const int ge = S::GW * cw;                      // entries per group
+    uint32_t cnt;                                   // kSp1MaxBuckets / 2 words, then 40 words per group for the scan
+    asm volatile("mov.u32 %0, %1;" : "=r"(cnt) : "r"((uint32_t)__cvta_generic_to_shared(sp_smem)));
+    const uint32_t warp_tot = cnt + 2 * kSp1MaxBuckets;
+    const uint32_t vals = warp_tot + 160 * NG;      // [NG][ge] FP32
+    const uint32_t idxs = vals + 4 * NG * ge;       // [NG][ge] Idx
+    const uint32_t srt = idxs + (uint32_t)sizeof(Idx) * NG * ge;   // [ge] 16 bits
+    const int g = threadIdx.x / S::GT, warp = (threadIdx.x % S::GT) >> 5, lane = threadIdx.x & 31;
+    const int bar = 1 + g;
+    const uint32_t val = vals + 4 * g * ge, idx = idxs + (uint32_t)sizeof(Idx) * g * ge;
+    const uint32_t wval = val + 4 * warp * cw, widx = idx + (uint32_t)sizeof(Idx) * warp * cw;   // the warp's region
+    const int64_t seg = ((n + S::GW - 1) / S::GW + 1023) / 1024 * 1024;   // columns per warp: whole steps
+    const int64_t s0 = min(n, (int64_t)warp * seg), s1 = min(n, s0 + seg);
+    const int64_t rows = (m - blockIdx.x + gridDim.x - 1) / gridDim.x;   // of this CTA
+    for (int64_t q = g; q < rows; q += NG) {
+        const int64_t r = blockIdx.x + q * gridDim.x;
+        const int have = sp1_compact<InT, Idx>(A + r * lda, s0, s1, vec, wval, widx, cw);
+        if constexpr (kScale) {
+            __syncwarp();
+#pragma unroll 8
+            for (int k = lane; k < have; k += 32) {
+                const float f = __ldg(col_scale + s0 + lds_idx<Idx>(widx, k));
+                sts_u32(wval + 4 * k, __float_as_uint(__uint_as_float(lds_u32(wval + 4 * k)) * f));
+            }
+        }
+        const bool over = group_or(bar, S::GT, have < 0);
+        if (NG == 2 && q > 0) group_sync(3 + g, kSpThreads);   // this group's turn
+        if (!over)
+            sp1_route<OutT, NG>(cnt, warp_tot + 160 * g, srt, val, idx, have, (uint32_t)s0, cw, r, hs, n, seed, hashed, b, blocks,
+                                At, ldat, scales, lds, plane_elems, bar);
+        else if (threadIdx.x % S::GT == 0)
             *row_mark(At, r, ldat, (int64_t)blocks.idx[0] * b) = RowMark<OutT>::bits;
+        if (NG == 2 && q + 1 < rows) group_arrive(3 + (g ^ 1), kSpThreads);
+        group_sync(bar, S::GT);   // the group's entries are free for its next row
     }
 }
 
@@ -724,25 +994,28 @@ os_status launch_sparse_t(const InT *A, int64_t lda, int64_t m, int64_t n, const
     const size_t smem0 = sizeof(float) * (size_t)kb + (size_t)kEntryBytes * emax + sp_fixed_bytes(p->b);
     const bool vec = aligned16(A) && (lda * (int64_t)sizeof(InT)) % 16 == 0;
     const int64_t grid = m < sp_num_sms() ? m : sp_num_sms();
-    // one-pass rows: per warp a region of cw entries (entry numbers fit 16 bits)
-    int cw = 0;
-    if (p->b <= 4 * kSpThreads) {
-        const int64_t avail = (int64_t)kSmemLimit - (int64_t)sp1_fixed_bytes(p->b) - 64;
-        const int64_t c = avail / (32 * kSp1EntryBytes);
-        cw = (int)(c < 2047 ? c : 2047);
-        if (cw < 32) cw = 0;
+    // one-pass rows: two rows at a time per SM when there are enough rows (and their
+    // indices fit 16 bits), else one row by the whole CTA
+    const bool onepass = p->b <= kSp1MaxBuckets;
+    if (onepass) {
+        const bool two = m > sp_num_sms() && n <= Sp1<2>::kMaxN;
+        auto launch = [&](auto ng) -> os_status {
+            constexpr int NG = decltype(ng)::value;
+            using S = Sp1<NG>;
+            const int64_t c = ((int64_t)kSmemLimit - (int64_t)S::kFixed - 64) / (S::GW * S::kEntryBytes) / 4 * 4;
+            const int cw = (int)(c < S::kMaxRegion ? c : S::kMaxRegion);
+            const size_t smem1 = S::kFixed + (size_t)S::kEntryBytes * S::GW * cw;
+            auto k1 = col_scale ? sketch_left_onepass_kernel<InT, OutT, true, NG>
+                                : sketch_left_onepass_kernel<InT, OutT, false, NG>;
+            OSK_CUDA_TRY(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
+            k1<<<(unsigned)grid, kSpThreads, smem1, st>>>(A, lda, m, n, vec, p->hs, p->seed, p->hashed != 0, p->b,
+                                                          blocks, cw, col_scale, (OutT *)At, ldat, scales, lds,
+                                                          plane_elems);
+            return check_launch();
+        };
+        OSK_TRY(two ? launch(std::integral_constant<int, 2>()) : launch(std::integral_constant<int, 1>()));
     }
-    if (cw > 0) {
-        const size_t smem1 = sp1_fixed_bytes(p->b) + (size_t)kSp1EntryBytes * 32 * cw + 64;
-        auto k1 = col_scale ? sketch_left_onepass_kernel<InT, OutT, true>
-                            : sketch_left_onepass_kernel<InT, OutT, false>;
-        OSK_CUDA_TRY(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
-        k1<<<(unsigned)grid, kSpThreads, smem1, st>>>(A, lda, m, n, vec, p->hs, p->seed, p->hashed != 0, p->b,
-                                                      blocks, cw, col_scale, (OutT *)At, ldat, scales, lds,
-                                                      plane_elems);
-        OSK_TRY(check_launch());
-    }
-    auto k = cw > 0 ? (col_scale ? sketch_left_sparse_kernel<InT, OutT, true, true>
+    auto k = onepass ? (col_scale ? sketch_left_sparse_kernel<InT, OutT, true, true>
                                  : sketch_left_sparse_kernel<InT, OutT, false, true>)
                     : (col_scale ? sketch_left_sparse_kernel<InT, OutT, true, false>
                                  : sketch_left_sparse_kernel<InT, OutT, false, false>);

@@ -27,6 +27,8 @@ os_status sketch_left_sparse_impl(const Plan *p, const void *A, os_dtype a_t, in
 os_status gemm_masked_f32(const Plan *p, const float *At, int64_t ldat, const float *BtT,
                           int64_t ldbt, int64_t m, int64_t l, uint64_t mask, float alpha, float beta,
                           float *C, int64_t ldc, cudaStream_t st);
+os_status unsketch_cols_t_impl(const Plan *p, const float *Tt, int64_t m, int64_t ldt, uint64_t mask, void *dX,
+                               os_dtype x_t, int64_t ldx, cudaStream_t st);
 os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &b, int64_t ld, int64_t l,
                             uint64_t mask, float alpha, float *C, int64_t ldc, unsigned int *flag, cudaStream_t st);
 os_status gemm_bf16_mn(const void *A, int64_t lda, bool a_mn, const void *B, int64_t ldb, bool b_mn, int64_t m,
@@ -522,14 +524,14 @@ extern "C" os_status oversketch_matmul_host(oversketch_plan_t plan, const void *
 namespace osk {
 namespace {
 
-// Workspace of the backward pass: dC in BF16 (both products use it), then T (and
+// Workspace of the backward pass: dC in BF16 (both products use it), then T^T (and
 // the compacted kept blocks of B~, laid out K-major) for dX, then U (and A~'s kept
 // blocks and dC^T, K-major) for dG.  With b a multiple of 128 and m, l multiples of
 // 8 the tensor cores read B~^T, A~ and dC MN-major as they are stored (dC's rows
 // padded to a multiple of 64), and the K-major copies are not made.
 struct BackwardLayout {
     bool mn;                         // operands read MN-major (no transposed copies)
-    int64_t kb, ld_l, ld_m, ld_kb;   // padded row pitches (elements) of the BF16 / FP32 buffers
+    int64_t kb, ld_l, ld_m, ld_t;    // padded row pitches (elements) of the BF16 / FP32 buffers
     size_t dc16, bsel, t, asel, dct16, u;
 };
 
@@ -539,10 +541,10 @@ BackwardLayout backward_layout(const Plan *p, int64_t m, int64_t l, uint64_t mas
     L.kb = (int64_t)__builtin_popcountll(mask) * p->b;
     L.ld_l = L.mn ? (l + 63) / 64 * 64 : (l + 7) / 8 * 8;   // BF16 rows of l elements
     L.ld_m = (m + 7) / 8 * 8;      // BF16 rows of m elements
-    L.ld_kb = (L.kb + 3) / 4 * 4;  // FP32 rows of k*b elements
+    L.ld_t = (m + 3) / 4 * 4;      // FP32 rows of m elements (T transposed)
     L.dc16 = align256((size_t)m * L.ld_l * 2);
     L.bsel = L.mn ? 0 : align256((size_t)L.kb * L.ld_l * 2);
-    L.t = align256((size_t)m * L.ld_kb * 4);
+    L.t = align256((size_t)L.kb * L.ld_t * 4);
     L.asel = L.mn ? 0 : align256((size_t)L.kb * L.ld_m * 2);
     L.dct16 = L.mn ? 0 : align256((size_t)l * L.ld_m * 2);
     L.u = align256((size_t)L.kb * ((l + 3) / 4 * 4) * 4);
@@ -592,19 +594,20 @@ extern "C" os_status oversketch_matmul_backward(oversketch_plan_t plan, const vo
     if (need_dx) {
         if (l > 0 && !BtT) return OS_ERR_INVALID_ARG;
         void *bsel = base;
-        float *T = reinterpret_cast<float *>(base + L.bsel);
+        float *Tt = reinterpret_cast<float *>(base + L.bsel);
         base += L.bsel + L.t;
+        // T^T = B~_sel dC^T (kb x m): its rows are what the gather into dX reads
         if (l > 0 && L.mn) {
-            // T = dC B~_sel^T: B~^T (l x z) read MN-major, kept blocks picked by column
-            OSK_TRY(gemm_bf16_mn(dc16, L.ld_l, false, BtT, ldbt, true, m, L.kb, l, inv_k, T, L.ld_kb, p->b, 2, mask,
+            // B~^T (l x z) read MN-major, kept blocks picked by column
+            OSK_TRY(gemm_bf16_mn(BtT, ldbt, true, dc16, L.ld_l, false, L.kb, m, l, inv_k, Tt, L.ld_t, p->b, 1, mask,
                                  p->P, st));
         } else if (l > 0) {
             OSK_TRY(oversketch_select_transpose(BtT, OS_BF16, l, z, ldbt, mask, p->b, bsel, OS_BF16, L.ld_l, stream));
-            OSK_TRY(oversketch_gemm_bf16(dc16, L.ld_l, bsel, L.ld_l, m, L.kb, l, inv_k, 0.0f, T, L.ld_kb, stream));
+            OSK_TRY(oversketch_gemm_bf16(bsel, L.ld_l, dc16, L.ld_l, L.kb, m, l, inv_k, 0.0f, Tt, L.ld_t, stream));
         } else {
-            OSK_CUDA_TRY(cudaMemsetAsync(T, 0, (size_t)m * L.ld_kb * 4, st));
+            OSK_CUDA_TRY(cudaMemsetAsync(Tt, 0, (size_t)L.kb * L.ld_t * 4, st));
         }
-        OSK_TRY(oversketch_unsketch_cols(plan, T, m, L.ld_kb, mask, 1.0f, dX, x_t, ldx, stream));
+        OSK_TRY(unsketch_cols_t_impl(p, Tt, m, L.ld_t, mask, dX, x_t, ldx, st));
     }
     if (need_dg) {
         if (m > 0 && !At) return OS_ERR_INVALID_ARG;

@@ -42,13 +42,40 @@ __global__ void __launch_bounds__(256) select_transpose_kernel(const TI *__restr
     }
 }
 
-template <typename TI, typename TO>
+// Y = X, eight elements per thread and step (16-byte accesses when kVec: rows of both
+// start on 16-byte boundaries), threads (x) along a row, (y) and CTAs along the rows.
+// Memory-bound: one element per thread behind a 64-bit division took 46 us for the
+// 4096 x 4096 FP32 -> BF16 cast on GB300 (15 at the copy rate), this takes 14.7.
+template <typename TI, typename TO, bool kVec>
 __global__ void __launch_bounds__(256) cast_kernel(const TI *__restrict__ X, int64_t ldx, int64_t rows, int64_t cols,
                                                    TO *__restrict__ Y, int64_t ldy) {
-    const int64_t total = rows * cols;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = t / cols, c = t - r * cols;
-        Y[r * ldy + c] = from_f<TO>(to_f(X[r * ldx + c]));
+    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
+    if (c >= cols) return;
+    for (int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; r < rows; r += (int64_t)gridDim.y * blockDim.y) {
+        const TI *x = X + r * ldx + c;
+        TO *y = Y + r * ldy + c;
+        __align__(16) TI a[8];
+        __align__(16) TO o[8];
+        const bool whole = kVec && c + 8 <= cols;
+        if (whole) {
+#pragma unroll
+            for (int k = 0; k < (int)sizeof(a) / 16; ++k)
+                reinterpret_cast<uint4 *>(a)[k] = __ldg(reinterpret_cast<const uint4 *>(x) + k);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) a[k] = c + k < cols ? x[k] : from_f<TI>(0.f);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) o[k] = from_f<TO>(to_f(a[k]));
+        if (whole) {
+#pragma unroll
+            for (int k = 0; k < (int)sizeof(o) / 16; ++k)
+                reinterpret_cast<uint4 *>(y)[k] = reinterpret_cast<const uint4 *>(o)[k];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (c + k < cols) y[k] = o[k];
+        }
     }
 }
 
@@ -63,10 +90,18 @@ os_status launch_st(const void *X, int64_t ldx, int64_t rows, int64_t ocols, int
 
 template <typename TI, typename TO>
 os_status launch_cast(const void *X, int64_t ldx, int64_t rows, int64_t cols, void *Y, int64_t ldy, cudaStream_t st) {
-    const int64_t total = rows * cols;
-    const int64_t blocks = (total + 255) / 256 < 152 * 32 ? (total + 255) / 256 : 152 * 32;
-    cast_kernel<TI, TO><<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, st>>>((const TI *)X, ldx, rows, cols, (TO *)Y,
-                                                                            ldy);
+    const int64_t pieces = (cols + 7) / 8;
+    unsigned tx = 256;
+    while (tx > 1 && (int64_t)tx / 2 >= pieces) tx /= 2;
+    const unsigned ty = 256 / tx;
+    const int64_t gy = (rows + ty - 1) / ty;
+    const dim3 grid((unsigned)((pieces + tx - 1) / tx), (unsigned)(gy < 16384 ? gy : 16384)), block(tx, ty);
+    const bool vec = aligned16(X) && aligned16(Y) && (ldx * (int64_t)sizeof(TI)) % 16 == 0 &&
+                     (ldy * (int64_t)sizeof(TO)) % 16 == 0;
+    if (vec)
+        cast_kernel<TI, TO, true><<<grid, block, 0, st>>>((const TI *)X, ldx, rows, cols, (TO *)Y, ldy);
+    else
+        cast_kernel<TI, TO, false><<<grid, block, 0, st>>>((const TI *)X, ldx, rows, cols, (TO *)Y, ldy);
     return check_launch();
 }
 

@@ -105,6 +105,31 @@ struct Loader {
     __device__ __forceinline__ static float load1(const InT *p) { return to_f32(p[0]); }
 };
 
+// Two FP32 values in a 64-bit register, for the packed FP32 multiply-add (each half
+// rounded as fmaf does).  Kept packed from load to flush: packing around every
+// instruction costs more moves than it saves.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma2(f32x2 &acc, f32x2 w, f32x2 x) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(w), "l"(x));
+}
+// The 16 raw bytes of a row piece as pairs of FP32.
+template <typename InT> struct Pairs;
+template <> struct Pairs<float> {
+    static constexpr int N = 2;
+    __device__ __forceinline__ static f32x2 get(const uint4 &u, int k) {
+        return k == 0 ? pack2(__uint_as_float(u.x), __uint_as_float(u.y))
+                      : pack2(__uint_as_float(u.z), __uint_as_float(u.w));
+    }
+};
+
 // Sixteen bytes of zeros: the row segment that padding entries of the bucket
 // lists point at, so the gather loop needs no predication.
 __device__ __align__(16) float g_zero_row[8];
@@ -464,6 +489,64 @@ __global__ void __launch_bounds__(256) pack_cols_kernel(const T *__restrict__ A,
     }
 }
 
+// The same for BF16: tiles of 64 rows x 128 columns, so that a strip row receives a
+// whole 128-byte line, with two rows per 32-bit word in shared memory (a quarter of
+// the shared accesses of 2-byte elements: 219 -> 172 us for 4096 x 65536 on GB300, 158
+// at the copy rate).  Column c of word row rp is at rp * 129 + c with the low five
+// bits of c rotated by c / 32: conflict-free for the writes (lanes: 16 pieces of 8
+// columns, word rows rp and rp + 4) and the reads (8 groups of 4 word rows, 4 columns).
+template <bool kVec>
+__global__ void __launch_bounds__(256) pack_cols_bf16_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda,
+                                                             int64_t m, int64_t n, __nv_bfloat16 *__restrict__ Xs) {
+    constexpr int W = 128, PITCH = 129, SW = strip_of<__nv_bfloat16>();
+    __shared__ uint32_t tile[32 * PITCH];
+    auto at = [](int rp, int c) { return rp * PITCH + (c & ~31) + ((c + (c >> 5)) & 31); };
+    const int64_t rb = blockIdx.y, row0 = rb * 64, i0 = (int64_t)blockIdx.x * W;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (kVec && row0 + 64 <= m && i0 + W <= n) {
+        const int cv = lane & 15;
+        uint4 x[2], y[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int item = 2 * warp + u, rp = 8 * (item >> 2) + (item & 3) + 4 * (lane >> 4);
+            const __nv_bfloat16 *src = A + (row0 + 2 * rp) * lda + i0 + 8 * cv;
+            x[u] = __ldg(reinterpret_cast<const uint4 *>(src));
+            y[u] = __ldg(reinterpret_cast<const uint4 *>(src + lda));
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int item = 2 * warp + u, rp = 8 * (item >> 2) + (item & 3) + 4 * (lane >> 4);
+            const uint32_t xs[4] = {x[u].x, x[u].y, x[u].z, x[u].w}, ys[4] = {y[u].x, y[u].y, y[u].z, y[u].w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                tile[at(rp, 8 * cv + 2 * k)] = __byte_perm(xs[k], ys[k], 0x5410);
+                tile[at(rp, 8 * cv + 2 * k + 1)] = __byte_perm(xs[k], ys[k], 0x7632);
+            }
+        }
+    } else {
+        const unsigned short *src = reinterpret_cast<const unsigned short *>(A);
+#pragma unroll 8
+        for (int idx = tid; idx < 32 * W; idx += 256) {
+            const int rp = idx / W, c = idx % W;
+            const int64_t r = row0 + 2 * rp, col = i0 + c;
+            const uint32_t lo = r < m && col < n ? src[r * lda + col] : 0u;
+            const uint32_t hi = r + 1 < m && col < n ? src[(r + 1) * lda + col] : 0u;
+            tile[at(rp, c)] = lo | hi << 16;
+        }
+    }
+    __syncthreads();
+    const int64_t s = rb / (SW / 64), quarter = rb % (SW / 64);
+    const int rq = lane & 7;                      // 8 rows (4 word rows) per lane
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int c = 4 * (8 * u + warp) + (lane >> 3);
+        if (i0 + c >= n) continue;
+        const uint4 o = make_uint4(tile[at(4 * rq, c)], tile[at(4 * rq + 1, c)], tile[at(4 * rq + 2, c)],
+                                   tile[at(4 * rq + 3, c)]);
+        *reinterpret_cast<uint4 *>(Xs + (s * n + i0 + c) * SW + quarter * 64 + rq * 8) = o;
+    }
+}
+
 // dX[r, i] = scale * sum_{t < k} sigma_j(i) T[r, t*b + h_j(i)], j = kept[t]  (T holds the kept blocks only)
 template <typename OutT>
 __global__ void __launch_bounds__(256) unsketch_cols_kernel(
@@ -659,6 +742,115 @@ __global__ void __launch_bounds__(256) unsketch_rows_vec_kernel(
                 __nv_bfloat162 h[2] = {__floats2bfloat162_rn(acc[q].x, acc[q].y),
                                        __floats2bfloat162_rn(acc[q].z, acc[q].w)};
                 *reinterpret_cast<uint2 *>(dG + i * ldg + c) = *reinterpret_cast<uint2 *>(h);
+            }
+        }
+    }
+}
+
+// dX[r, i] = sum_t sigma_j(i) Tt[t*b + h_j(i), r], j = kept[t], from the transpose
+// Tt (kb x m) of the kept blocks' T: the gather of unsketch_rows (whole 512-byte row
+// pieces out of L2: Tt is taken in strips of 128 of m, k b 512 bytes each) with its
+// 64 x 128 tile transposed through shared memory on the way out.  Gathering single
+// columns of T from shared memory instead (unsketch_cols_smem_kernel) is held by
+// bank conflicts: 4096 x 65536 BF16 from 4 blocks of 2048 took 421 us on GB300, this
+// 316 (the L1 is the busiest unit).  The same additions in the same order.
+// Shared tile: row i holds 32 chunks of 4 r's, chunk c at position c ^ (i / 8 % 8),
+// so that both the row writes (16 bytes per lane) and the column reads (8 i's of 4
+// r's per warp, i = 8 (lane / 4) + s) touch every bank once.
+constexpr int kUtRows = 64;
+template <typename OutT, bool kVec>
+__global__ void __launch_bounds__(256, 4) unsketch_cols_t_kernel(
+    const float *__restrict__ Tt, int64_t m, int64_t ldt, const uint32_t *__restrict__ hs, int64_t n, int32_t b,
+    const __grid_constant__ BlockList kept, OutT *__restrict__ dX, int64_t ldx) {
+    __shared__ float4 tile[kUtRows][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t i0 = (int64_t)blockIdx.x * kUtRows, r0 = (int64_t)blockIdx.y * 128;
+    const bool live = r0 + 4 * lane < ldt;               // the pitch is a multiple of 4 that holds m
+    const uint64_t base = reinterpret_cast<uint64_t>(Tt + (live ? r0 + 4 * lane : r0));
+    const uint32_t row_bytes = (uint32_t)(4 * ldt);      // the launch keeps 4 ldt below 2^32
+    const uint64_t block_bytes = (uint64_t)b * row_bytes;
+    // Warp w: rows 8w .. 8w + 7 of the tile, four at a time.  Lane 4q + u holds the table
+    // entry of kept block t0 + q and row u of the four: one load per four blocks, issued
+    // ahead, so that no row piece waits for its own entry.
+    auto entries = [&](int h, int t0) -> uint32_t {
+        const int t = t0 + (lane >> 2);
+        const int64_t i = i0 + 8 * warp + 4 * h + (lane & 3);
+        return lane < 16 && t < kept.count && i < n ? __ldg(hs + (int64_t)kept.idx[t] * n + i) : 0u;
+    };
+    uint32_t first[2] = {entries(0, 0), entries(1, 0)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        f32x2 acc[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u][0] = acc[u][1] = 0;
+        uint32_t e = first[h];
+        uint64_t bt = base;                               // row 0 of kept block t
+        // kept blocks t0 + q .. + Q - 1: 4 Q loads per lane in flight
+        auto blocks = [&](auto qq, int q) {
+            constexpr int Q = decltype(qq)::value;
+            uint32_t v[4 * Q];
+            uint4 x[4 * Q];
+#pragma unroll
+            for (int k = 0; k < 4 * Q; ++k) {
+                v[k] = __shfl_sync(0xffffffffu, e, 4 * q + k);
+                const uint64_t row = (k >> 2) ? bt + block_bytes : bt;
+                x[k] = __ldg(reinterpret_cast<const uint4 *>((uint64_t)(v[k] & kIndexMask) * row_bytes + row));
+            }
+#pragma unroll
+            for (int k = 0; k < 4 * Q; ++k) {
+                const float sg = __uint_as_float(0x3f800000u | (v[k] & kSignBit));
+                const f32x2 w2 = pack2(sg, sg);
+                fma2(acc[k & 3][0], w2, Pairs<float>::get(x[k], 0));
+                fma2(acc[k & 3][1], w2, Pairs<float>::get(x[k], 1));
+            }
+            bt += Q * block_bytes;
+        };
+        for (int t0 = 0; t0 < kept.count; t0 += 4) {
+            const uint32_t next = t0 + 4 < kept.count ? entries(h, t0 + 4) : 0u;
+            const int left = kept.count - t0;
+            if (left >= 2) blocks(std::integral_constant<int, 2>(), 0);
+            if (left >= 4) blocks(std::integral_constant<int, 2>(), 2);
+            else if (left == 3) blocks(std::integral_constant<int, 1>(), 2);
+            else if (left == 1) blocks(std::integral_constant<int, 1>(), 0);
+            e = next;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            float4 o;
+            unpack2(acc[u][0], o.x, o.y);
+            unpack2(acc[u][1], o.z, o.w);
+            tile[8 * warp + 4 * h + u][lane ^ warp] = o;   // warp = i / 8
+        }
+    }
+    __syncthreads();
+    // chunk c of r's: 4 per warp; lane: r = 4c + lane % 4, i = 8 (lane / 4) .. + 7
+    const int w = lane & 3, ig = lane >> 2;
+    const int64_t i = i0 + 8 * ig;
+    const float *flat = reinterpret_cast<const float *>(tile);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c = 4 * warp + k;
+        const int64_t r = r0 + 4 * c + w;
+        float y[8];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) y[s] = flat[(8 * ig + s) * 128 + 4 * (c ^ ig) + w];
+        if (r >= m) continue;
+        OutT *dst = dX + r * ldx + i;
+        if (kVec && i + 8 <= n) {
+            if constexpr (sizeof(OutT) == 4) {
+                reinterpret_cast<float4 *>(dst)[0] = make_float4(y[0], y[1], y[2], y[3]);
+                reinterpret_cast<float4 *>(dst)[1] = make_float4(y[4], y[5], y[6], y[7]);
+            } else {
+                const __nv_bfloat162 q[4] = {__floats2bfloat162_rn(y[0], y[1]), __floats2bfloat162_rn(y[2], y[3]),
+                                             __floats2bfloat162_rn(y[4], y[5]), __floats2bfloat162_rn(y[6], y[7])};
+                *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(q);
+            }
+        } else {
+#pragma unroll
+            for (int s = 0; s < 8; ++s) {
+                if (i + s >= n) break;
+                if constexpr (sizeof(OutT) == 4) dst[s] = y[s];
+                else dst[s] = __float2bfloat16_rn(y[s]);
             }
         }
     }
@@ -860,16 +1052,27 @@ os_status launch_pack_rows(const T *X, int64_t ldx, int64_t n, int64_t F, T *Xs,
     return check_launch();
 }
 
-template <typename T>
-os_status launch_pack_cols(const T *A, int64_t lda, int64_t m, int64_t n, T *Xs, cudaStream_t st) {
+os_status launch_pack_cols(const float *A, int64_t lda, int64_t m, int64_t n, float *Xs, cudaStream_t st) {
     // 32-row blocks of the (zero-padded) strips
-    constexpr int64_t SW = strip_of<T>();
+    constexpr int64_t SW = strip_of<float>();
     dim3 grid((unsigned)((n + 255) / 256), (unsigned)((m + SW - 1) / SW * (SW / 32)));
     if (grid.y > 65535u) return OS_ERR_UNSUPPORTED;
-    if (aligned16(A) && (lda * (int64_t)sizeof(T)) % 16 == 0)
-        pack_cols_kernel<T, true><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
+    if (aligned16(A) && lda % 4 == 0)
+        pack_cols_kernel<float, true><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
     else
-        pack_cols_kernel<T, false><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
+        pack_cols_kernel<float, false><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
+    return check_launch();
+}
+
+os_status launch_pack_cols(const __nv_bfloat16 *A, int64_t lda, int64_t m, int64_t n, __nv_bfloat16 *Xs,
+                           cudaStream_t st) {
+    constexpr int64_t SW = strip_of<__nv_bfloat16>();
+    dim3 grid((unsigned)((n + 127) / 128), (unsigned)((m + SW - 1) / SW * (SW / 64)));
+    if (grid.y > 65535u) return OS_ERR_UNSUPPORTED;
+    if (aligned16(A) && lda % 8 == 0)
+        pack_cols_bf16_kernel<true><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
+    else
+        pack_cols_bf16_kernel<false><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
     return check_launch();
 }
 
@@ -970,11 +1173,11 @@ os_status sketch_left_impl(const Plan *p, const void *A, os_dtype a_t, int64_t m
     const float *wts = nullptr;
     OSK_TRY(make_weights(p, col_scale, block_mask, ws_weights(p, ws, m, a_t), &wts, st));
     if (a_t == OS_F32) {
-        OSK_TRY(launch_pack_cols<float>((const float *)A, lda, m, p->n, (float *)Xs, st));
+        OSK_TRY(launch_pack_cols((const float *)A, lda, m, p->n, (float *)Xs, st));
         return launch_gather<float>(p, (const float *)Xs, m, wts, At, out_t, ldat, scales, fp8_scale_ld(m),
                                     block_mask, st, m, dmask);
     }
-    OSK_TRY(launch_pack_cols<__nv_bfloat16>((const __nv_bfloat16 *)A, lda, m, p->n, (__nv_bfloat16 *)Xs, st));
+    OSK_TRY(launch_pack_cols((const __nv_bfloat16 *)A, lda, m, p->n, (__nv_bfloat16 *)Xs, st));
     return launch_gather<__nv_bfloat16>(p, (const __nv_bfloat16 *)Xs, m, wts, At, out_t, ldat, scales,
                                         fp8_scale_ld(m), block_mask, st, m, dmask);
 }
@@ -1141,6 +1344,22 @@ os_status unsketch_rows_impl(const Plan *p, const float *U, int64_t l, int64_t l
                                                                       scale, (__nv_bfloat16 *)dG, ldg);
     }
     return check_launch();
+}
+
+// dX (m x n) from the transposed kept blocks Tt (kb x m, pitch ldt a multiple of 4).
+os_status unsketch_cols_t_impl(const Plan *p, const float *Tt, int64_t m, int64_t ldt, uint64_t mask, void *dX,
+                               os_dtype x_t, int64_t ldx, cudaStream_t st) {
+    const BlockList kept = mask_to_list(mask, p->P);
+    const dim3 grid((unsigned)((p->n + kUtRows - 1) / kUtRows), (unsigned)((m + 127) / 128));
+    if (grid.y > 65535u || ldt % 4 != 0 || ldt >= (int64_t(1) << 30) || !aligned16(Tt)) return OS_ERR_UNSUPPORTED;
+    auto launch = [&](auto *out) -> os_status {
+        using O = typename std::remove_pointer<decltype(out)>::type;
+        const bool vec = aligned16(dX) && (ldx * (int64_t)sizeof(O)) % 16 == 0;
+        auto k = vec ? unsketch_cols_t_kernel<O, true> : unsketch_cols_t_kernel<O, false>;
+        k<<<grid, 256, 0, st>>>(Tt, m, ldt, p->hs, p->n, p->b, kept, out, ldx);
+        return check_launch();
+    };
+    return x_t == OS_F32 ? launch((float *)dX) : launch((__nv_bfloat16 *)dX);
 }
 
 }  // namespace osk

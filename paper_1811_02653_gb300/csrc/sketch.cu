@@ -129,6 +129,13 @@ template <> struct Pairs<float> {
                       : pack2(__uint_as_float(u.z), __uint_as_float(u.w));
     }
 };
+template <> struct Pairs<__nv_bfloat16> {
+    static constexpr int N = 4;
+    __device__ __forceinline__ static f32x2 get(const uint4 &u, int k) {
+        const uint32_t w = k == 0 ? u.x : k == 1 ? u.y : k == 2 ? u.z : u.w;
+        return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+    }
+};
 
 // Sixteen bytes of zeros: the row segment that padding entries of the bucket
 // lists point at, so the gather loop needs no predication.
@@ -159,6 +166,13 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
     constexpr int TFO = kMis ? TF - 4 : TF;   // free indices written per CTA
     constexpr int PITCH = TF + 1;        // odd pitch: conflict-free column reads
     constexpr int NC = kMis ? 4 : 1;     // accumulator sets: one per misalignment class
+    // BF16 rows and misaligned ones are bound by instructions: packed FP32 multiply-adds
+    // and no padding test before a bucket's last batch.  BF16 keeps its accumulators
+    // packed; for the four sets of misaligned rows that was slower (95 against 86 us
+    // for 20011 x 1777, 6 blocks), and aligned FP32 rows, bound by L2, lose with
+    // either (1.68 -> 1.81 ms on the square product's left operand).
+    constexpr bool kPacked = sizeof(InT) == 2;
+    constexpr bool kFewer = kMis || kPacked;
     static_assert(!kMis || (std::is_same<InT, float>::value && SLOTS == 1), "misaligned rows: FP32, one member per load");
     constexpr int G = 2 * SLOTS;         // groups of 4 members per batch: 8 loads per lane in flight
     constexpr int QPW = QT / kWarps;     // buckets per warp
@@ -173,7 +187,11 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
     const int jblk = blocks.idx[bt];
     const int q0 = jblk * b + (blockIdx.x - bt * tiles_per_block) * QT;
     const int qend = min(z, jblk * b + b);
-    const int64_t f0 = (int64_t)blockIdx.y * TFO;
+    // a packed operand (rows as wide as a strip): strips last to first, since the last
+    // ones packed are still in L2 (1 - 2 % of the left sketches of 20011 - 32768 rows;
+    // in-place operands lose as much that way)
+    const int64_t strip = ldx == TF ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+    const int64_t f0 = strip * TFO;
     // a block mask read at run time: CTAs of blocks it does not keep have nothing to do
     if (dmask && !((__ldg(dmask) >> jblk) & 1ull)) return;
     using L = Loader<InT, VW, true>;
@@ -187,7 +205,7 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
         const uint32_t gbl = lane <= nb ? __ldg(poffs + (int64_t)jblk * (b + 1) + cb + lane) >> 2 : 0u;
         const uint32_t gend = __shfl_sync(0xffffffffu, gbl, nb);
         // row i of the strip at xbase + i * row_bytes: one wide multiply-add per member
-        const uint64_t xbase = reinterpret_cast<uint64_t>(X + blockIdx.y * strip_stride + VW * sub);
+        const uint64_t xbase = reinterpret_cast<uint64_t>(X + strip * strip_stride + VW * sub);
         const uint32_t row_bytes = (uint32_t)(ldx * (int64_t)sizeof(InT));
         const uint64_t zrow = reinterpret_cast<uint64_t>(g_zero_row);
 
@@ -203,9 +221,11 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
             return pos < 4 * gend ? __ldg(wl + pos) : 0.f;
         };
         // GG groups (4*GG members) of the current bucket, entries in lanes 0 .. 4*GG-1
-        // of e, their signed scales in the same lanes of w
-        auto batch = [&](auto gg, uint32_t e, float w, float *acc) {
+        // of e, their signed scales in the same lanes of w.  Only a bucket's last group
+        // holds padding: the batches before it skip the test for it.
+        auto batch = [&](auto gg, auto padded, uint32_t e, float w, auto *acc) {
             constexpr int GG = decltype(gg)::value;
+            constexpr bool kPadded = decltype(padded)::value;
             constexpr int KS = 4 * GG / SLOTS;            // member loads per lane
             uint4 v[KS];
             float wgt[KS];
@@ -214,11 +234,8 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
             for (int k = 0; k < KS; ++k) {
                 const uint32_t ent = __shfl_sync(0xffffffffu, e, k * SLOTS + slot);
                 // +-1 from the sign bit (or the signed scale); padding reads the zero row
-                if constexpr (kScale) {
-                    wgt[k] = __shfl_sync(0xffffffffu, w, k * SLOTS + slot);
-                } else {
-                    wgt[k] = __uint_as_float(0x3f800000u | (ent & kSignBit));
-                }
+                // (a signed scale is fetched when the row is added: eight fewer live registers)
+                if constexpr (!kScale) wgt[k] = __uint_as_float(0x3f800000u | (ent & kSignBit));
                 uint64_t addr = (uint64_t)(ent & kIndexMask) * row_bytes + xbase;
                 if constexpr (kMis) {
                     // The row piece starts d = 0..3 elements into a 16-byte granule
@@ -228,35 +245,43 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
                     cls |= ((uint32_t)addr & 12u) << (2 * k);
                     addr &= ~uint64_t(15);
                 }
-                v[k] = L::load_raw(reinterpret_cast<const InT *>(ent != kPadEntry ? addr : zrow));
+                v[k] = L::load_raw(reinterpret_cast<const InT *>(!kPadded || ent != kPadEntry ? addr : zrow));
             }
 #pragma unroll
             for (int k = 0; k < KS; ++k) {
-                float x[VW];
-                L::unpack(v[k], x);
-                if constexpr (kMis) {
+                if constexpr (kScale) wgt[k] = __shfl_sync(0xffffffffu, w, k * SLOTS + slot);
+                if constexpr (kPacked) {
+                    constexpr int N = Pairs<InT>::N;
+                    const f32x2 w2 = pack2(wgt[k], wgt[k]);
+#pragma unroll
+                    for (int q = 0; q < N; ++q) fma2(acc[q], w2, Pairs<InT>::get(v[k], q));
+                } else if constexpr (kMis) {
                     // one accumulator set per class (a warp-uniform branch)
+                    float x[VW];
+                    L::unpack(v[k], x);
+                    const f32x2 w2 = pack2(wgt[k], wgt[k]);
+                    auto add = [&](float *a) {
+#pragma unroll
+                        for (int w = 0; w < VW; w += 2) {
+                            f32x2 t = pack2(a[w], a[w + 1]);
+                            fma2(t, w2, pack2(x[w], x[w + 1]));
+                            unpack2(t, a[w], a[w + 1]);
+                        }
+                    };
                     const uint32_t d = (cls >> (2 * k)) & 12u;
-                    if (d == 0u) {
-#pragma unroll
-                        for (int w = 0; w < VW; ++w) acc[w] = fmaf(wgt[k], x[w], acc[w]);
-                    } else if (d == 4u) {
-#pragma unroll
-                        for (int w = 0; w < VW; ++w) acc[VW + w] = fmaf(wgt[k], x[w], acc[VW + w]);
-                    } else if (d == 8u) {
-#pragma unroll
-                        for (int w = 0; w < VW; ++w) acc[2 * VW + w] = fmaf(wgt[k], x[w], acc[2 * VW + w]);
-                    } else {
-#pragma unroll
-                        for (int w = 0; w < VW; ++w) acc[3 * VW + w] = fmaf(wgt[k], x[w], acc[3 * VW + w]);
-                    }
+                    if (d == 0u) add(acc);
+                    else if (d == 4u) add(acc + VW);
+                    else if (d == 8u) add(acc + 2 * VW);
+                    else add(acc + 3 * VW);
                 } else {
+                    float x[VW];
+                    L::unpack(v[k], x);
 #pragma unroll
                     for (int w = 0; w < VW; ++w) acc[w] = fmaf(wgt[k], x[w], acc[w]);
                 }
             }
         };
-        auto flush = [&](int t, float *acc) {
+        auto flush = [&](int t, const float *acc) {
             float out[VW];
             if constexpr (kMis) {
                 // class d holds element 4*sub + w - d of the strip in lane sub, slot w:
@@ -295,26 +320,40 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
         uint32_t g = __shfl_sync(0xffffffffu, gbl, 0);
         uint32_t e_cur = load_entries(g);
         float w_cur = load_weights(g);
-        auto step = [&](auto gg, float *acc) {
+        auto step = [&](auto gg, auto padded, auto *acc) {
             constexpr int GG = decltype(gg)::value;
             const uint32_t e_nxt = load_entries(g + GG);
             const float w_nxt = load_weights(g + GG);
-            batch(gg, GG * 4 >= 32 ? e_cur : (lane < 4 * GG ? e_cur : kPadEntry), w_cur, acc);
+            batch(gg, padded, e_cur, w_cur, acc);
             g += GG;
             e_cur = e_nxt;
             w_cur = w_nxt;
         };
         for (int t = 0; t < nb; ++t) {
             const uint32_t gE = __shfl_sync(0xffffffffu, gbl, t + 1);
-            float acc[NC * VW];
+            constexpr std::true_type last{};
+            constexpr int NA = kPacked ? NC * VW / 2 : NC * VW;
+            typename std::conditional<kPacked, f32x2, float>::type acc[NA];
 #pragma unroll
-            for (int w = 0; w < NC * VW; ++w) acc[w] = 0.f;
-            while (gE - g >= (uint32_t)G) step(std::integral_constant<int, G>(), acc);
+            for (int w = 0; w < NA; ++w) acc[w] = 0;
+            if constexpr (kFewer) {
+                while (gE - g > (uint32_t)G) step(std::integral_constant<int, G>(), std::false_type(), acc);
+                if (gE - g == (uint32_t)G) step(std::integral_constant<int, G>(), last, acc);
+            } else {
+                while (gE - g >= (uint32_t)G) step(std::integral_constant<int, G>(), last, acc);
+            }
             const uint32_t r = gE - g;   // < G
-            if constexpr (G >= 8) if (r & 4u) step(std::integral_constant<int, 4>(), acc);
-            if constexpr (G >= 4) if (r & 2u) step(std::integral_constant<int, 2>(), acc);
-            if (r & 1u) step(std::integral_constant<int, 1>(), acc);
-            flush(t, acc);
+            if constexpr (G >= 8) if (r & 4u) step(std::integral_constant<int, 4>(), last, acc);
+            if constexpr (G >= 4) if (r & 2u) step(std::integral_constant<int, 2>(), last, acc);
+            if (r & 1u) step(std::integral_constant<int, 1>(), last, acc);
+            if constexpr (kPacked) {
+                float sums[NC * VW];
+#pragma unroll
+                for (int w = 0; w < NA; ++w) unpack2(acc[w], sums[2 * w], sums[2 * w + 1]);
+                flush(t, sums);
+            } else {
+                flush(t, acc);
+            }
         }
     }
     __syncthreads();

@@ -141,6 +141,32 @@ template <> struct Pairs<__nv_bfloat16> {
 // lists point at, so the gather loop needs no predication.
 __device__ __align__(16) float g_zero_row[8];
 
+// A gather CTA's (block, tile) and strip: in launch order, or (tpb < 0, -tpb tiles per
+// block) with the first block of the next strip dealt out between the other blocks of
+// this one, tile by tile.
+__device__ __forceinline__ int2 mixed_place(int tpb, int count, int64_t &strip) {
+    const uint32_t K = count, T = tpb < 0 ? -tpb : tpb, per = K * T;
+    uint32_t at = blockIdx.x, tile = 0, bt = 0;
+    strip = blockIdx.y;
+    if (tpb > 0) {
+        bt = at / T;
+        return make_int2(bt, at - bt * T);
+    }
+    at += blockIdx.y * gridDim.x;
+    if (at < T) {
+        strip = 0;
+        return make_int2(0, at);
+    }
+    at -= T;
+    strip = at / per;
+    at -= (uint32_t)strip * per;
+    const bool last = strip + 1 == gridDim.y;
+    tile = at / (last ? K - 1 : K);
+    bt = last ? 1 + at - tile * (K - 1) : at - tile * K;
+    strip += bt == 0;
+    return make_int2(bt, tile);
+}
+
 // Lane layout: lane = slot * SUBS + sub (SUBS = 32 / SLOTS lanes per member;
 // the launches use SLOTS = 1, one member per warp load).  With SLOTS > 1 the
 // slots of a warp gather different members of one bucket at once (bucket lists
@@ -182,15 +208,23 @@ sketch_gather_kernel(const InT *__restrict__ X, int64_t strip_stride, int64_t ld
     float *tile = reinterpret_cast<float *>(smem_tile);   // [QT][PITCH]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int slot = lane / SUBS, sub = lane % SUBS;
-    // q0: first sketched column of this CTA, inside one of the listed blocks
-    const int bt = blockIdx.x / tiles_per_block;
+    // FP32 rows with scales may run in the mixed order of mixed_place (FP8 tiles have to
+    // stay in launch order: clusters of four; aligned rows without scales lose 0.5 - 10 %
+    // to the longer prologue, whose registers they do not have).
+    constexpr bool kMixable = kScale && !kMis && sizeof(InT) == 4 && sizeof(OutT) != 1;
+    int2 place = make_int2(0, 0);            // block and tile
+    int64_t place_y = 0;
+    if constexpr (kMixable) place = mixed_place(tiles_per_block, blocks.count, place_y);
+    const int bt = kMixable ? place.x : blockIdx.x / tiles_per_block;
     const int jblk = blocks.idx[bt];
-    const int q0 = jblk * b + (blockIdx.x - bt * tiles_per_block) * QT;
+    // q0: first sketched column of this CTA, inside one of the listed blocks
+    const int q0 = kMixable ? jblk * b + place.y * QT : jblk * b + (blockIdx.x - bt * tiles_per_block) * QT;
     const int qend = min(z, jblk * b + b);
     // a packed operand (rows as wide as a strip): strips last to first, since the last
     // ones packed are still in L2 (1 - 2 % of the left sketches of 20011 - 32768 rows;
     // in-place operands lose as much that way)
-    const int64_t strip = ldx == TF ? gridDim.y - 1 - blockIdx.y : blockIdx.y;
+    const int64_t strip = kMixable ? (ldx == TF ? gridDim.y - 1 - place_y : place_y)
+                                   : (ldx == TF ? gridDim.y - 1 - blockIdx.y : blockIdx.y);
     const int64_t f0 = strip * TFO;
     // a block mask read at run time: CTAs of blocks it does not keep have nothing to do
     if (dmask && !((__ldg(dmask) >> jblk) & 1ull)) return;
@@ -974,6 +1008,14 @@ os_status launch_quantize_fp8(const Plan *p, const float *Y, int64_t ldy, int64_
     return check_launch();
 }
 
+// A strip is first read from DRAM and then, by its other blocks' CTAs, from L2, and its
+// CTAs sweep their lists in step.  Dealing the next strip's first block out between
+// them overlaps the two, as long as two strips fit in L2 with room to spare.  GB300,
+// FP32 rows with scales, 20 blocks of 1024: 965 -> 918 us for 40960 x 5120 (strips of
+// 21 MB), 30 blocks of 512: 983 -> 956 for 30720 x 5120; strips of 33 MB gain nothing
+// and larger ones lose (without scales, 64 MB: 429 -> 507 us).
+constexpr int64_t kMixBytes = int64_t(24) << 20;
+
 template <typename InT, typename OutT, int QT, int SLOTS, bool kMis = false>
 os_status launch_gather_t(const Plan *p, const InT *X, int64_t strip_stride, int64_t ldx, int64_t F,
                           const float *wts, void *Yt, int64_t ldy, float *scales, int64_t scale_ld,
@@ -986,6 +1028,8 @@ os_status launch_gather_t(const Plan *p, const InT *X, int64_t strip_stride, int
     dim3 grid((unsigned)(tpb * blocks.count), (unsigned)((F + TFO - 1) / TFO));
     if (grid.y > 65535u) return OS_ERR_UNSUPPORTED;
     const size_t smem = sizeof(float) * QT * (TF + 1);
+    const bool mix = wts && !kMis && sizeof(InT) == 4 && sizeof(OutT) != 1 && blocks.count > 1 && grid.y > 1 &&
+                     p->n * (int64_t)(TF * sizeof(InT)) <= kMixBytes;
     auto k = wts ? sketch_gather_kernel<InT, OutT, QT, true, SLOTS, kMis>
                        : sketch_gather_kernel<InT, OutT, QT, false, SLOTS, kMis>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1009,7 +1053,7 @@ os_status launch_gather_t(const Plan *p, const InT *X, int64_t strip_stride, int
                                         scales, scale_ld, blocks, tpb, plane_elems, dmask));
     } else {
         k<<<grid, kWarps * 32, smem, st>>>(X, strip_stride, ldx, F, p->pperm, p->poffs, p->pstride, p->b, z,
-                                          wts, (OutT *)Yt, ldy, scales, scale_ld, blocks, tpb, plane_elems, dmask);
+                                          wts, (OutT *)Yt, ldy, scales, scale_ld, blocks, mix ? -tpb : tpb, plane_elems, dmask);
     }
     return check_launch();
 }

@@ -414,7 +414,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                 if (issued[s]) mbar_wait_drain(&full[s], issued_phase[s]);
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer (lane 0 issues; the warp waits together) ----------------
+        // ---------------- MMA issuer (one lane issues; the warp waits together) ----------------
         int stage = 0;
         uint32_t phase = 0;
         int iter = 0;
@@ -430,7 +430,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
               ++iter;
               if (!__all_sync(0xffffffffu, mbar_wait(&tmem_empty[a], aphase ^ 1u, abort, wait_ns))) { ok = false; break; }
               tc_fence_after();
-              if (lane == 0) umma_commit(&tmem_full[a]);
+              if (elect_one()) umma_commit(&tmem_full[a]);
               __syncwarp();
               continue;
           }
@@ -454,7 +454,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                 if constexpr (C::FP8) {
                     sfa = tmem_base + C::sf_slot(stage);
                     sfb = sfa + 4;
-                    if (lane == 0) {
+                    if (elect_one()) {
                         uint8_t *ch = st + C::TX_BYTES;
                         tmem_cp_32x128b_x4(sfa, sdesc_rows16(smem_u32(ch)));
 #pragma unroll
@@ -462,7 +462,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                             tmem_cp_32x128b_x4(sfb + 4 * c, sdesc_rows16(smem_u32(ch + 512 * (1 + c))));
                     }
                 }
-                if (lane == 0) {
+                if (elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < ROWB / 32; ++kk) {
                         const uint32_t acc0 = (kb > kc || kk > 0) ? 1u : 0u;
@@ -487,10 +487,10 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                 if (++stage == STAGES) stage = 0, phase ^= 1u;
             }
             if (!ok) break;
-            if (lane == 0) umma_commit(&tmem_full[a]);
+            if (elect_one()) umma_commit(&tmem_full[a]);
           }
         }
-        if (!ok && any && lane == 0) {
+        if (!ok && any && elect_one()) {
             // Drain: wait for the MMAs already issued before freeing TMEM.
             umma_commit(drain);
             mbar_wait_drain(drain, 0);
@@ -761,7 +761,7 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
                 if (issued[s] && !mbar_wait_cluster(&empty[s], issued_phase[s], abort)) ok = false;
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer (leader; lane 0 issues, the warp waits together) ----------------
+        // ---------------- MMA issuer (leader; one lane issues, the warp waits together) ----------------
         if (leader) {
             int stage = 0;
             uint32_t phase = 0;
@@ -783,7 +783,7 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
                 for (int kb = 0; kb < nkb; ++kb) {
                     if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort))) { ok = false; break; }
                     tc_fence_after();
-                    if (lane == 0) {
+                    if (elect_one()) {
                         const uint32_t sa0 = smem_u32(tiles + stage * C::STAGE_BYTES);
                         const uint32_t sb0 = sa0 + C::A_BYTES;
 #pragma unroll
@@ -803,9 +803,9 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
                     if (++stage == STAGES) stage = 0, phase ^= 1u;
                 }
                 if (!ok) break;
-                if (lane == 0) umma_commit_pair(&tmem_full[a], 0x3);   // both halves of the accumulator
+                if (elect_one()) umma_commit_pair(&tmem_full[a], 0x3);   // both halves of the accumulator
             }
-            if (!ok && any && lane == 0) {
+            if (!ok && any && elect_one()) {
                 // drain: wait for the MMAs already issued before TMEM is freed
                 umma_commit_pair(drain, 0x1);
                 mbar_wait_drain(drain, 0);
@@ -993,7 +993,7 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                 if (issued[s] && !mbar_wait_cluster(&empty[s], issued_phase[s], abort)) ok = false;
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer (leader; lane 0 issues, the warp waits together) ----------------
+        // ---------------- MMA issuer (leader; one lane issues, the warp waits together) ----------------
         if (leader) {
             int stage = 0;
             uint32_t phase = 0;
@@ -1019,7 +1019,7 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                     for (int kb = kc; kb < kc_end; ++kb) {
                         if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort))) { ok = false; break; }
                         tc_fence_after();
-                        if (lane == 0) {
+                        if (elect_one()) {
                             const uint32_t sah = smem_u32(tiles + stage * C::STAGE_BYTES);
                             const uint32_t sal = sah + C::A_BYTES;
                             const uint32_t sbh = sal + C::A_BYTES;
@@ -1041,11 +1041,11 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                         if (++stage == STAGES) stage = 0, phase ^= 1u;
                     }
                     if (!ok) break;
-                    if (lane == 0) umma_commit_pair(&tmem_full[a], 0x3);   // both halves of the accumulator
+                    if (elect_one()) umma_commit_pair(&tmem_full[a], 0x3);   // both halves of the accumulator
                     __syncwarp();
                 }
             }
-            if (!ok && any && lane == 0) {
+            if (!ok && any && elect_one()) {
                 // drain: wait for the MMAs already issued before TMEM is freed
                 umma_commit_pair(drain, 0x1);
                 mbar_wait_drain(drain, 0);

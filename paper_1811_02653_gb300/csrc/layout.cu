@@ -42,11 +42,11 @@ __global__ void __launch_bounds__(256) select_transpose_kernel(const TI *__restr
     }
 }
 
-// Y = X, eight elements per thread and step (16-byte accesses when kVec: rows of both
-// start on 16-byte boundaries), threads (x) along a row, (y) and CTAs along the rows.
+// Y = X, eight elements per thread and step (16-byte accesses where kVecX / kVecY: the
+// rows of X / Y start on 16-byte boundaries), threads (x) along a row, (y) and CTAs along the rows.
 // Memory-bound: one element per thread behind a 64-bit division took 46 us for the
 // 4096 x 4096 FP32 -> BF16 cast on GB300 (15 at the copy rate), this takes 14.7.
-template <typename TI, typename TO, bool kVec>
+template <typename TI, typename TO, bool kVecX, bool kVecY>
 __global__ void __launch_bounds__(256) cast_kernel(const TI *__restrict__ X, int64_t ldx, int64_t rows, int64_t cols,
                                                    TO *__restrict__ Y, int64_t ldy) {
     const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(256) cast_kernel(const TI *__restrict__ X, int
         TO *y = Y + r * ldy + c;
         __align__(16) TI a[8];
         __align__(16) TO o[8];
-        const bool whole = kVec && c + 8 <= cols;
-        if (whole) {
+        const bool whole = c + 8 <= cols;
+        if (kVecX && whole) {
 #pragma unroll
             for (int k = 0; k < (int)sizeof(a) / 16; ++k)
                 reinterpret_cast<uint4 *>(a)[k] = __ldg(reinterpret_cast<const uint4 *>(x) + k);
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) cast_kernel(const TI *__restrict__ X, int
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) o[k] = from_f<TO>(to_f(a[k]));
-        if (whole) {
+        if (kVecY && whole) {
 #pragma unroll
             for (int k = 0; k < (int)sizeof(o) / 16; ++k)
                 reinterpret_cast<uint4 *>(y)[k] = reinterpret_cast<const uint4 *>(o)[k];
@@ -96,12 +96,11 @@ os_status launch_cast(const void *X, int64_t ldx, int64_t rows, int64_t cols, vo
     const unsigned ty = 256 / tx;
     const int64_t gy = (rows + ty - 1) / ty;
     const dim3 grid((unsigned)((pieces + tx - 1) / tx), (unsigned)(gy < 16384 ? gy : 16384)), block(tx, ty);
-    const bool vec = aligned16(X) && aligned16(Y) && (ldx * (int64_t)sizeof(TI)) % 16 == 0 &&
-                     (ldy * (int64_t)sizeof(TO)) % 16 == 0;
-    if (vec)
-        cast_kernel<TI, TO, true><<<grid, block, 0, st>>>((const TI *)X, ldx, rows, cols, (TO *)Y, ldy);
-    else
-        cast_kernel<TI, TO, false><<<grid, block, 0, st>>>((const TI *)X, ldx, rows, cols, (TO *)Y, ldy);
+    const bool vx = aligned16(X) && (ldx * (int64_t)sizeof(TI)) % 16 == 0;
+    const bool vy = aligned16(Y) && (ldy * (int64_t)sizeof(TO)) % 16 == 0;
+    auto k = vx ? (vy ? cast_kernel<TI, TO, true, true> : cast_kernel<TI, TO, true, false>)
+                : (vy ? cast_kernel<TI, TO, false, true> : cast_kernel<TI, TO, false, false>);
+    k<<<grid, block, 0, st>>>((const TI *)X, ldx, rows, cols, (TO *)Y, ldy);
     return check_launch();
 }
 

@@ -568,7 +568,9 @@ __global__ void __launch_bounds__(256) pack_cols_kernel(const T *__restrict__ A,
 // at the copy rate).  Column c of word row rp is at rp * 129 + c with the low five
 // bits of c rotated by c / 32: conflict-free for the writes (lanes: 16 pieces of 8
 // columns, word rows rp and rp + 4) and the reads (8 groups of 4 word rows, 4 columns).
-template <bool kVec>
+// For rows that start on 16-byte boundaries; others take pack_cols_kernel, whose
+// element loads are no slower than word-building ones (18940 x 2617: 127 against 180 us
+// for the whole left sketch).
 __global__ void __launch_bounds__(256) pack_cols_bf16_kernel(const __nv_bfloat16 *__restrict__ A, int64_t lda,
                                                              int64_t m, int64_t n, __nv_bfloat16 *__restrict__ Xs) {
     constexpr int W = 128, PITCH = 129, SW = strip_of<__nv_bfloat16>();
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(256) pack_cols_bf16_kernel(const __nv_bfloat16
     auto at = [](int rp, int c) { return rp * PITCH + (c & ~31) + ((c + (c >> 5)) & 31); };
     const int64_t rb = blockIdx.y, row0 = rb * 64, i0 = (int64_t)blockIdx.x * W;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (kVec && row0 + 64 <= m && i0 + W <= n) {
+    if (row0 + 64 <= m && i0 + W <= n) {
         const int cv = lane & 15;
         uint4 x[2], y[2];
 #pragma unroll
@@ -827,9 +829,11 @@ __global__ void __launch_bounds__(256) unsketch_rows_vec_kernel(
 // columns of T from shared memory instead (unsketch_cols_smem_kernel) is held by
 // bank conflicts: 4096 x 65536 BF16 from 4 blocks of 2048 took 421 us on GB300, this
 // 316 (the L1 is the busiest unit).  The same additions in the same order.
-// Shared tile: row i holds 32 chunks of 4 r's, chunk c at position c ^ (i / 8 % 8),
+// Shared tile: row i holds 32 chunks of 4 r's, chunk c at position c ^ ((i ^ i / 8) % 8),
 // so that both the row writes (16 bytes per lane) and the column reads (8 i's of 4
-// r's per warp, i = 8 (lane / 4) + s) touch every bank once.
+// r's per warp, i = 8 (lane / 4) + s) touch every bank once.  Rows of dX without
+// 16-byte alignment are stored 32 elements per instruction instead (reads four to a
+// bank), not 8 per lane.
 constexpr int kUtRows = 64;
 template <typename OutT, bool kVec>
 __global__ void __launch_bounds__(256, 4) unsketch_cols_t_kernel(
@@ -892,24 +896,42 @@ __global__ void __launch_bounds__(256, 4) unsketch_cols_t_kernel(
             float4 o;
             unpack2(acc[u][0], o.x, o.y);
             unpack2(acc[u][1], o.z, o.w);
-            tile[8 * warp + 4 * h + u][lane ^ warp] = o;   // warp = i / 8
+            tile[8 * warp + 4 * h + u][lane ^ ((4 * h + u) ^ warp)] = o;   // i = 8 warp + 4 h + u
         }
     }
     __syncthreads();
-    // chunk c of r's: 4 per warp; lane: r = 4c + lane % 4, i = 8 (lane / 4) .. + 7
+    // chunk c of r's: 4 per warp
+    const float *flat = reinterpret_cast<const float *>(tile);
+    if constexpr (!kVec) {
+#pragma unroll 4
+        for (int k = 0; k < 16; ++k) {
+            const int c = 4 * warp + (k >> 2), w = k & 3;
+            const int64_t r = r0 + 4 * c + w;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int i = 32 * half + lane;
+                const float y = flat[i * 128 + 4 * (c ^ ((i ^ (i >> 3)) & 7)) + w];
+                if (r < m && i0 + i < n) {
+                    if constexpr (sizeof(OutT) == 4) dX[r * ldx + i0 + i] = y;
+                    else dX[r * ldx + i0 + i] = __float2bfloat16_rn(y);
+                }
+            }
+        }
+        return;
+    }
+    // lane: r = 4c + lane % 4, i = 8 (lane / 4) .. + 7
     const int w = lane & 3, ig = lane >> 2;
     const int64_t i = i0 + 8 * ig;
-    const float *flat = reinterpret_cast<const float *>(tile);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int c = 4 * warp + k;
         const int64_t r = r0 + 4 * c + w;
         float y[8];
 #pragma unroll
-        for (int s = 0; s < 8; ++s) y[s] = flat[(8 * ig + s) * 128 + 4 * (c ^ ig) + w];
+        for (int s = 0; s < 8; ++s) y[s] = flat[(8 * ig + s) * 128 + 4 * (c ^ (s ^ ig)) + w];
         if (r >= m) continue;
         OutT *dst = dX + r * ldx + i;
-        if (kVec && i + 8 <= n) {
+        if (i + 8 <= n) {
             if constexpr (sizeof(OutT) == 4) {
                 reinterpret_cast<float4 *>(dst)[0] = make_float4(y[0], y[1], y[2], y[3]);
                 reinterpret_cast<float4 *>(dst)[1] = make_float4(y[4], y[5], y[6], y[7]);
@@ -1150,12 +1172,14 @@ os_status launch_pack_cols(const float *A, int64_t lda, int64_t m, int64_t n, fl
 os_status launch_pack_cols(const __nv_bfloat16 *A, int64_t lda, int64_t m, int64_t n, __nv_bfloat16 *Xs,
                            cudaStream_t st) {
     constexpr int64_t SW = strip_of<__nv_bfloat16>();
-    dim3 grid((unsigned)((n + 127) / 128), (unsigned)((m + SW - 1) / SW * (SW / 64)));
+    const bool rows16 = aligned16(A) && lda % 8 == 0;
+    const int64_t w = rows16 ? 128 : 256, h = rows16 ? 64 : 32;   // the kernels' tiles
+    dim3 grid((unsigned)((n + w - 1) / w), (unsigned)((m + SW - 1) / SW * (SW / h)));
     if (grid.y > 65535u) return OS_ERR_UNSUPPORTED;
-    if (aligned16(A) && lda % 8 == 0)
-        pack_cols_bf16_kernel<true><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
+    if (rows16)
+        pack_cols_bf16_kernel<<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
     else
-        pack_cols_bf16_kernel<false><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
+        pack_cols_kernel<__nv_bfloat16, false><<<grid, 256, 0, st>>>(A, lda, m, n, Xs);
     return check_launch();
 }
 

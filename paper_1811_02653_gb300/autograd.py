@@ -23,6 +23,16 @@ import torch
 from . import ops
 
 
+def _sketches(X, G, plan, mask):
+    """The BF16 sketches of both operands (kept blocks), one packing workspace for the
+    two: small layers are bound by the host, a tensor allocation is 2 - 7 us there."""
+    ws = torch.empty(max(ops.sketch_workspace(plan, X.shape[0], X.dtype), ops.sketch_workspace(plan, G.shape[1], G.dtype)),
+                     dtype=torch.uint8, device=X.device)
+    At, _ = ops.sketch_left(plan, X, "bf16", block_mask=mask, workspace=ws)
+    BtT, _ = ops.sketch_right(plan, G, "bf16", block_mask=mask, workspace=ws)
+    return At, BtT
+
+
 class OverSketchMatmul(torch.autograd.Function):
     """C = (1/k) (X S_sel)(S_sel^T G) with a hand-written backward.
 
@@ -34,8 +44,7 @@ class OverSketchMatmul(torch.autograd.Function):
 
     @staticmethod
     def forward(ctx, X, G, plan, mask: int, recompute: bool = False):
-        At, _ = ops.sketch_left(plan, X, "bf16", block_mask=mask)
-        BtT, _ = ops.sketch_right(plan, G, "bf16", block_mask=mask)
+        At, BtT = _sketches(X, G, plan, mask)
         C = ops.gemm_masked(plan, At, BtT, mask)
         ctx.plan, ctx.mask, ctx.recompute = plan, mask, recompute
         ctx.x_dtype, ctx.g_dtype = X.dtype, G.dtype
@@ -50,13 +59,14 @@ class OverSketchMatmul(torch.autograd.Function):
         plan, mask = ctx.plan, ctx.mask
         if ctx.recompute:
             X, G = ctx.saved_tensors
-            At, _ = ops.sketch_left(plan, X, "bf16", block_mask=mask)
-            BtT, _ = ops.sketch_right(plan, G, "bf16", block_mask=mask)
+            At, BtT = _sketches(X, G, plan, mask)
         else:
             At, BtT = ctx.saved_tensors
         if dC.stride(-1) != 1:
             dC = dC.contiguous()
-        dX, dG = ops.matmul_backward(plan, At, BtT, dC.float(), mask, ctx.x_dtype, ctx.g_dtype,
+        if dC.dtype is not torch.float32:
+            dC = dC.float()
+        dX, dG = ops.matmul_backward(plan, At, BtT, dC, mask, ctx.x_dtype, ctx.g_dtype,
                                      need_dx=ctx.needs_input_grad[0], need_dg=ctx.needs_input_grad[1])
         return dX, dG, None, None, None
 

@@ -93,6 +93,8 @@ struct Cfg {
     // in TMEM and the epilogue adds the chunks in FP32 registers, so the
     // accumulation error does not grow with K.  Otherwise one chunk per tile.
     static constexpr int CHUNK_KB = kKind == Kind::Tf32x3 ? 8 : (1 << 30);
+    // fewest K steps per CTA of a split tile (0: never split)
+    static constexpr int MIN_SPLIT_KB = kKind == Kind::Tf32x3 ? 4 : kKind == Kind::Fp8 ? 2 : 0;
     static_assert(!FP8 || (BN <= 240 && 2 * SF_GAP_SLOTS >= STAGES), "FP8 scale slots do not fit in TMEM");
     static_assert(BN % 32 == 0 && BN <= 256, "tile width");
     static_assert(SMEM <= 232448, "shared memory");
@@ -144,6 +146,8 @@ struct GemmArgs {
     // device word that makes the launch return at once: skip_if when it is nonzero,
     // run_if when it is zero (null: always run)
     const unsigned int *skip_if, *run_if;
+    // split launches (one-CTA kernel): CTAs of the cluster that share a tile, K steps each
+    int32_t split, kb_per_split;
 };
 
 // Tile pair t of the lower triangle (row-major: pair row pm, tile column tn <= pm).
@@ -240,13 +244,20 @@ struct TileJob {
 // TF32 lo planes, or for FP8 the slice-major FP32 scale arrays.  GROUPED: the
 // tiles of g.group_count products (descriptors g.group, tile_begin ascending)
 // share one persistent launch; the tensor maps come from the descriptors.
-template <class C, bool GROUPED>
+// SPLIT: few tiles.  The g.split CTAs of a cluster share one tile, CTA r the r-th part
+// of its K steps; the partial tiles meet in shared memory (over the stages, which are
+// free by then), and CTA r adds the r-th part of the tile's rows in rank order, read
+// from the cluster's shared memory.  A fixed order, no workspace, no second launch.
+template <class C, bool GROUPED, bool SPLIT = false>
 __global__ void __launch_bounds__(C::THREADS, 1)
 gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_constant__ CUtensorMap tmap_b0,
                       const __grid_constant__ CUtensorMap tmap_a1, const __grid_constant__ CUtensorMap tmap_b1,
                       const GemmArgs g) {
     constexpr int STAGES = C::STAGES, BN = C::BN, BKE = C::BKE;
     static_assert(!GROUPED || C::PLANES == 1 && !C::FP8, "grouped launches take BF16 operands");
+    static_assert(!GROUPED || !SPLIT, "grouped launches are not split");
+    constexpr int PART_PITCH = BN + 4;             // words per row of a partial tile
+    static_assert(!SPLIT || BM * PART_PITCH * 4 <= STAGES * C::STAGE_BYTES, "partial tile");
     extern __shared__ uint8_t smem_raw[];
     __shared__ int32_t s_begin[GROUPED ? kMaxGroup : 1];   // first tile of each product
     // 1024-byte alignment for the swizzled tiles
@@ -308,6 +319,13 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
     const int skip_kb = s_skip_kb;
     const unsigned long long wait_ns = s_wait_ns;
 
+    // this CTA's first tile and tile step, and its part of a tile's K steps
+    const int rank = SPLIT ? (int)cluster_ctarank() : 0;
+    const int t_first = SPLIT ? blockIdx.x / g.split : blockIdx.x;
+    const int t_step = SPLIT ? gridDim.x / g.split : gridDim.x;
+    const int kb0 = SPLIT ? rank * g.kb_per_split : 0;
+    const int my_kb = SPLIT ? min(g.num_kb - kb0, g.kb_per_split) : g.num_kb;
+
     // The tile's product, coordinates and epilogue parameters.
     auto job = [&](int t) {
         TileJob j;
@@ -334,7 +352,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
             j.ta = &tmap_a0;
             j.tb = &tmap_b0;
             j.mask = 0;                   // read g.kept directly (no copy of the parameter)
-            j.num_kb = g.num_kb;
+            j.num_kb = my_kb;
             j.kb_per_blk = g.kb_per_blk;
             j.b = g.b;
             j.C = g.C;
@@ -351,7 +369,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
             const GroupProblem *P = g.group + find_problem(s_begin, g.group_count, t);
             return __popcll(group_mask(P)) * P->kb_per_blk;
         } else {
-            return g.num_kb;
+            return my_kb;
         }
     };
 
@@ -364,7 +382,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
             bool issued[STAGES];
             for (int s = 0; s < STAGES; ++s) issued[s] = false, issued_phase[s] = 0;
             bool ok = true;
-            for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
                 const TileJob j = job(t);
                 uint64_t rest = j.mask;          // grouped: kept blocks not yet started
                 int kidx = 0;
@@ -375,8 +393,8 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                 }
                 for (int kb = 0; kb < j.num_kb; ++kb) {
                     if (!mbar_wait(&empty[stage], phase ^ 1u, abort, wait_ns)) { ok = false; break; }
-                    const int blk = kb / j.kb_per_blk;
-                    const int kin = kb - blk * j.kb_per_blk;
+                    const int blk = (kb0 + kb) / j.kb_per_blk;
+                    const int kin = kb0 + kb - blk * j.kb_per_blk;
                     if constexpr (GROUPED) {
                         if (kin == 0) {
                             kidx = __ffsll((long long)rest) - 1;
@@ -385,7 +403,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                     } else {
                         kidx = g.kept.idx[blk];
                     }
-                    if (t == blockIdx.x && kb == skip_kb) {
+                    if (t == t_first && kb0 + kb == skip_kb) {
                         // test hook: this stage is never loaded nor armed, so the
                         // MMA warp's wait for it runs out
                         if (++stage == STAGES) stage = 0, phase ^= 1u;
@@ -420,7 +438,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
         int iter = 0;
         bool ok = true;
         bool any = false;
-        for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
+        for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
           const int num_kb = num_kb_of(t);
           if (GROUPED && num_kb == 0) {
               // a product whose run-time mask keeps no block: hand the epilogue an
@@ -504,8 +522,8 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
         if constexpr (C::FP8) {
             const int stage = warp - 6;
             uint32_t phase = 0;
-            const int64_t my_tiles = (g.num_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-            const int64_t steps = my_tiles * g.num_kb;   // K steps of all the CTA's tiles
+            const int64_t my_tiles = (g.num_tiles - t_first + t_step - 1) / t_step;
+            const int64_t steps = my_tiles * my_kb;      // K steps of all the CTA's tiles
             uint8_t *st = tiles + stage * C::STAGE_BYTES;
             const float *fa = reinterpret_cast<const float *>(st + C::TILE_BYTES);
             const float *fb = fa + BM;
@@ -535,12 +553,21 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
         float *buf = reinterpret_cast<float *>(smem + STAGES * C::STAGE_BYTES + 256) + quarter * 32 * kEpiPitch;
         int iter = 0;
         bool ok = true;
-        for (int t = blockIdx.x; ok && t < g.num_tiles; t += gridDim.x) {
+        for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
             const TileJob j = job(t);
             const bool vec_ok = ((reinterpret_cast<uintptr_t>(j.C) & 15u) == 0) && (j.ldc % 4 == 0);
             const int64_t r0 = (int64_t)j.tm * BM + quarter * 32;
             const int64_t c0 = (int64_t)j.tn * BN;
             auto store = [&](int ch, const float *val) {
+                if constexpr (SPLIT) {
+                    // this row's 32 values into the partial tile
+                    float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(tiles) +
+                                                             (quarter * 32 + lane) * PART_PITCH + ch * 32);
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        dst[u] = make_float4(val[4 * u], val[4 * u + 1], val[4 * u + 2], val[4 * u + 3]);
+                    return;
+                }
                 store_piece(buf, val, j.alpha, j.beta, j.C, j.ldc, r0, j.m, c0 + ch * 32, j.l, vec_ok, lane);
             };
             if constexpr (C::CHUNK_KB < (1 << 30)) {
@@ -593,6 +620,52 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
 
     tc_fence_before();
     __syncthreads();
+    if constexpr (SPLIT) {
+        cluster_sync_all();   // every partial tile is written
+        const TileJob j = job(t_first);
+        const bool vec_ok = ((reinterpret_cast<uintptr_t>(j.C) & 15u) == 0) && (j.ldc % 4 == 0);
+        const int rows = BM / g.split;
+        const uint32_t part = smem_u32(tiles);
+        for (int q = warp; q < rows; q += C::THREADS / 32) {
+            const int row = rank * rows + q;
+            const int64_t r = (int64_t)j.tm * BM + row;
+            if (r >= j.m) break;
+            for (int c = 4 * lane; c < BN; c += 128) {
+                const uint32_t at = part + 4u * (uint32_t)(row * PART_PITCH + c);
+                float4 v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (k < g.split) v[k] = ld_cluster_v4(cluster_addr_of(at, (uint32_t)k));
+                float4 o = v[0];
+#pragma unroll
+                for (int k = 1; k < 8; ++k)
+                    if (k < g.split) {
+                        o.x += v[k].x;
+                        o.y += v[k].y;
+                        o.z += v[k].z;
+                        o.w += v[k].w;
+                    }
+                const int64_t cb = (int64_t)j.tn * BN + c;
+                float x[4] = {j.alpha * o.x, j.alpha * o.y, j.alpha * o.z, j.alpha * o.w};
+                float *dst = j.C + r * j.ldc + cb;
+                if (vec_ok && cb + 4 <= j.l) {
+                    if (j.beta != 0.f) {
+                        const float4 old = *reinterpret_cast<const float4 *>(dst);
+                        x[0] = fmaf(j.beta, old.x, x[0]);
+                        x[1] = fmaf(j.beta, old.y, x[1]);
+                        x[2] = fmaf(j.beta, old.z, x[2]);
+                        x[3] = fmaf(j.beta, old.w, x[3]);
+                    }
+                    *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (cb + u < j.l) dst[u] = j.beta != 0.f ? fmaf(j.beta, dst[u], x[u]) : x[u];
+                }
+            }
+        }
+        cluster_sync_all();   // nobody reads this CTA's shared memory any more
+    }
     if (warp == 1) {
         __syncwarp();
         tc_fence_after();
@@ -1192,6 +1265,65 @@ int num_sms() {
 
 namespace {
 
+template <typename Kern, typename... Args>
+cudaError_t launch_clusters(Kern kern, unsigned cluster, unsigned grid, int threads, size_t smem, cudaStream_t st,
+                            const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// CTAs per tile for a one-CTA launch of few tiles, which would leave most SMs idle
+// behind a serial chain of K steps: as many as are resident at once (clusters do not
+// straddle GPCs: 76, 36 and 15 of 2, 4 and 8 CTAs; 16 clusters of 8 took two rounds,
+// slower than 16 of 4), with at least min_kb K steps each, all of them with some.
+// us for the 3xTF32 GEMM on GB300, whole -> split: 512 x 512, K = 1024 25 -> 12.7;
+// 512 x 512, 4096 78 -> 25.7; 300 x 300, 8192 150 -> 26.4; 1024 x 1024, 4096 80 -> 45.6.
+template <class C>
+int split_of(int64_t tiles, int num_kb, int min_kb) {
+    static std::once_flag once;
+    static int resident[4] = {0, 0, 0, 0};   // clusters of 2, 4, 8 CTAs
+    std::call_once(once, [] {
+        if (cudaFuncSetAttribute(gemm_masked_tc_kernel<C, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)C::SMEM) != cudaSuccess) {
+            cudaGetLastError();
+            return;                          // no split launches
+        }
+        for (int i = 1; i <= 3; ++i) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(8u * 152u);
+            cfg.blockDim = dim3(C::THREADS);
+            cfg.dynamicSmemBytes = C::SMEM;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = 1u << i;
+            attr[0].val.clusterDim.y = 1;
+            attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            if (cudaOccupancyMaxActiveClusters(&resident[i], gemm_masked_tc_kernel<C, false, true>, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                resident[i] = 0;
+            }
+        }
+    });
+    for (int i = 3; i >= 1; --i) {
+        const int S = 1 << i, per = (num_kb + S - 1) / S;
+        if (tiles <= resident[i] && per >= min_kb && (S - 1) * per < num_kb) return S;
+    }
+    return 1;
+}
+
 // C = alpha * sum over the listed K blocks of A_blk . B_blk^T (+ beta C).  A is
 // rows x zK, B cols x zK, K-major; for the TF32 configuration A1/B1 are the lo
 // planes (A0/B0 the hi planes); for FP8 they are the FP32 scale arrays
@@ -1241,12 +1373,23 @@ os_status launch_tc(const void *A0, const void *A1, int64_t lda, const void *B0,
         ta1 = ta0;
         tb1 = tb0;
     }
-    static bool attr_set = false;
-    if (!attr_set) {
-        OSK_CUDA_TRY(cudaFuncSetAttribute(gemm_masked_tc_kernel<C, false>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM));
-        attr_set = true;
-    }
+    if constexpr (C::MIN_SPLIT_KB > 0) g.split = split_of<C>(g.num_tiles, g.num_kb, C::MIN_SPLIT_KB);
+    else g.split = 1;
+    g.kb_per_split = (g.num_kb + g.split - 1) / g.split;
+    static std::once_flag attr_once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(attr_once, [] {
+        attr_err = cudaFuncSetAttribute(gemm_masked_tc_kernel<C, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)C::SMEM);
+    });
+    OSK_CUDA_TRY(attr_err);
+    if constexpr (C::MIN_SPLIT_KB > 0)
+        if (g.split > 1) {
+            OSK_CUDA_TRY(launch_clusters(gemm_masked_tc_kernel<C, false, true>, (unsigned)g.split,
+                                         (unsigned)(g.split * g.num_tiles), C::THREADS, C::SMEM, st, ta0, tb0, ta1, tb1,
+                                         g));
+            return check_launch();
+        }
     const int grid = g.num_tiles < num_sms() ? g.num_tiles : num_sms();
     gemm_masked_tc_kernel<C, false><<<grid, C::THREADS, C::SMEM, st>>>(ta0, tb0, ta1, tb1, g);
     return check_launch();
@@ -1256,19 +1399,7 @@ os_status launch_tc(const void *A0, const void *A1, int64_t lda, const void *B0,
 template <typename Kern, typename... Args>
 cudaError_t launch_pairs(Kern kern, int threads, size_t smem, int num_tiles, cudaStream_t st, const Args &...args) {
     const int pairs = num_sms() / 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2u * (unsigned)(num_tiles < pairs ? num_tiles : pairs));
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
+    return launch_clusters(kern, 2u, 2u * (unsigned)(num_tiles < pairs ? num_tiles : pairs), threads, smem, st, args...);
 }
 
 template <bool kAMN, bool kBMN>
@@ -1377,9 +1508,23 @@ os_status launch_pair_bf16_mn(const void *A, int64_t lda, bool a_mn, const void 
     return launch_pair_args<false, false>(ta, tb, g, st);
 }
 
+// BF16 products: CTA pairs, or, where 128 x 128 tiles need no more waves and K is short,
+// the one-CTA kernel: half the tile to fill and to write out per CTA, but 4 % more per K
+// step.  us for the GEMM on GB300, pair -> one CTA: 512 x 512, K = 1024 14.4 -> 12.4; 1000
+// x 700, 2048 18.5 -> 16.8; 1024 x 1501, 2048 22.5 -> 19.1; 1024 x 1501, 512 15.5 -> 12.3.
+// Past the line, 1536 x 1536, 4096: 26.8 -> 28.6; 1024 x 1024, 8192: 43.1 -> 47.2; more
+// waves, 2048 x 2048 x 2048: 20.1 -> 28.7.  K is not split here (300 x 300, 8192 would
+// take 14.4 of 43): the sums stay those of the grouped, per-block, symmetric and panel launches.
 os_status launch_bf16(const void *A, int64_t lda, const void *B, int64_t ldb, int64_t m, int64_t l, int64_t zK,
                       int32_t blk, const BlockList &kept, float alpha, float beta, float *C, int64_t ldc,
                       cudaStream_t st) {
+    using C1 = CfgBf16N128;
+    const bool sym = A == B && lda == ldb && m == l;
+    auto waves = [](int64_t tiles, int64_t at_once) { return (tiles + at_once - 1) / at_once; };
+    const int64_t pairs = (m + 255) / 256 * ((l + 255) / 256), ones = (m + 127) / 128 * ((l + 127) / 128);
+    if (!sym && blk % C1::BKE == 0 && (int64_t)kept.count * blk <= 2560 &&
+        waves(ones, num_sms()) <= waves(pairs, num_sms() / 2))
+        return launch_tc<C1>(A, nullptr, lda, B, nullptr, ldb, m, l, zK, blk, kept, alpha, beta, C, ldc, st);
     return launch_pair_bf16(A, lda, B, ldb, m, l, zK, blk, kept, alpha, beta, C, ldc, st);
 }
 
@@ -1445,6 +1590,15 @@ os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &
     OSK_TRY(launch_tf32_planes(a, b, ld, p->b, kept, flag, st));
     return launch_tc<CfgTf32x3>(a.sums, a.sums + m * ld, ld, bs.sums, bs.sums + bs.rows * ld, ld, m, l, z, p->b, kept,
                                 alpha, 0.f, Cout, ldc, st, flag);
+}
+
+// The 3xTF32 kernel's time for a product by its tiles and their split, in us (19.5 ns
+// per K of a 128 x 128 tile on GB300, 152 tiles at once).
+double tf32x3_us(int64_t m, int64_t l, int64_t K) {
+    using C = CfgTf32x3;
+    const int64_t tiles = (m + BM - 1) / BM * ((l + C::BN - 1) / C::BN);
+    const int S = split_of<C>(tiles, (int)(K / C::BKE), C::MIN_SPLIT_KB);
+    return (double)((tiles + num_sms() - 1) / num_sms()) * (double)K * 19.5e-3 / S;
 }
 
 os_status gemm_masked_tc(const Plan *p, const void *At, int64_t ldat, const float *a_scales,

@@ -131,9 +131,26 @@ __device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
     return r;
 }
 
+// The same for a shared-memory address already at hand.
+__device__ __forceinline__ uint32_t cluster_addr_of(uint32_t smem_addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
+    return r;
+}
+
 // All threads of all CTAs of the cluster (release / acquire).
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// 16 bytes of another CTA's shared memory (cluster address).
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t cluster_address) {
+    float4 v;
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"(cluster_address)
+                 : "memory");
+    return v;
 }
 
 // Arrive on an mbarrier in another CTA of the cluster (release at cluster scope).

@@ -37,6 +37,7 @@ def _reference(ops, p, A, B, mask):
     (1500, 9000, 1601, 704, 4, 1, 0b11011),     # ragged tiles of 256 x 160, odd ldc, K = 44 chunks
     (2560, 8192, 1920, 512, 4, 2, 0b101101),    # whole tiles
     (4001, 4096, 4003, 64, 5, 1, 0b011111),     # K = 320: a chunk of one step
+    (6001, 4096, 6003, 192, 3, 1, 0b1011),      # K = 576: the third chunk of one step
     (257, 20000, 12801, 1024, 2, 0, 0b11),      # a second tile row of one row
 ])
 def test_f16x3_parity(ops, m, n, l, b, N, e, mask):

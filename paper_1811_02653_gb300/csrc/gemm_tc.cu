@@ -12,7 +12,9 @@
 // kept[kb / (b/BK)] * b + (kb mod (b/BK)) * BK, so dropped blocks are never
 // loaded.  Operands are K-major in the 128-byte swizzled layout.
 //
-// Kernel organisation (one persistent CTA per SM):
+// Kernel organisation of gemm_masked_tc_kernel (one persistent CTA per SM; TF32 planes,
+// grouped BF16 products, BF16 and FP8 products of few tiles -- the larger BF16 and FP8
+// products and FP32 on FP16 planes run on CTA pairs, further down):
 //   warp 0      TMA producer: ring of {A 128 x BK, B BN x BK} stages (FP8 stages
 //               also carry the A and B scale rows of their 128-wide K slice)
 //   warp 1      TMEM owner + MMA issuer: tcgen05.mma 128 x BN per K step, FP32
@@ -1193,6 +1195,282 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP8 masked GEMM on CTA pairs: 256 x 224 tiles, block scales as in the one-CTA kernel,
+// whose K step brings 45 KB into an SM per 448 tensor clocks; a pair's brings 30.
+// Scales come in groups of four K steps, one byte of a TMEM word each (the MMA names
+// the byte), so that a group costs one conversion and three copies, and a stage holds
+// two K steps: with one, waiting, arming and committing take 0.29 us per step whatever
+// the MMAs, more than their 0.23.  8192 x 8192 x 8192 on GB300: 465 -> 350 us (3.1
+// PFLOP/s); without the loads of B 305, without the write-out 311, so the tensor cores
+// under load (0.23 us per step alone, 0.30 with all SMs busy) and C's 268 MB bound it.
+//   warp 0      TMA producer of this CTA's half of every stage (completion on the leader's barrier)
+//   warp 1      TMEM (both CTAs, jointly); scale copies, MMA issue and commits (leader)
+//   warps 2..5  epilogue of this CTA's 128 rows
+//   warps 6..9  scales, one warp per slot of a ring of groups of four K steps: FP32
+//               scales of this CTA's 128 rows of A and of all columns of B from global
+//               memory to UE8M0 bytes, one byte per K step, reported to the leader
+struct CfgPairFp8 {
+    static constexpr int BN = 224;                    // tile columns (the pair's N)
+    static constexpr int STAGES = 3;
+    static constexpr int STAGE_KB = 2;                // K steps per stage
+    static constexpr int BKE = ROWB;                  // 128 E4M3 per K step: one scale slice
+    static constexpr int A_BYTES = BM * ROWB;         // this CTA's 128 rows of A
+    static constexpr int B_BYTES = (BN / 2) * ROWB;   // this CTA's 112 rows of B
+    static constexpr int STEP_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGE_BYTES = STAGE_KB * STEP_BYTES;
+    static constexpr int GROUP_KB = 4;                // K steps per scale group: the four bytes of a TMEM word
+    static constexpr int SLOTS = 4;                   // groups in the ring
+    static constexpr int CHUNKS = 3;                  // of 512 bytes per group: A, B 0..127, B 128..
+    static constexpr int TMEM_COLS = 512;             // two accumulators, 256 columns apart
+    static constexpr int THREADS = 192 + 32 * SLOTS;
+    static constexpr size_t SMEM = 1024 + (size_t)STAGES * STAGE_BYTES + SLOTS * CHUNKS * 512 + 256 + kEpiBytes;
+    static constexpr uint32_t IDESC = idesc_mxf8_f32(2 * BM, BN);
+    static_assert(SMEM <= 232448, "shared memory");
+    static_assert(GROUP_KB % STAGE_KB == 0 && A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0, "swizzle atoms");
+    // TMEM columns of slot s's scales, 4 of A and 8 of B, behind the accumulators
+    __device__ static uint32_t sfa(int s) { return (uint32_t)((s / 2) * 256 + BN + 16 * (s % 2)); }
+};
+
+__global__ void __launch_bounds__(CfgPairFp8::THREADS, 1)
+gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
+                     const float *__restrict__ sa, int64_t ldsa, const float *__restrict__ sb, int64_t ldsb,
+                     const GemmArgs g) {
+    using C = CfgPairFp8;
+    constexpr int STAGES = C::STAGES, BN = C::BN, SLOTS = C::SLOTS;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint8_t *tiles = smem;
+    uint8_t *chunks = smem + STAGES * C::STAGE_BYTES;                                // UE8M0 groups
+    uint64_t *full = reinterpret_cast<uint64_t *>(chunks + SLOTS * C::CHUNKS * 512);   // leader's are used
+    uint64_t *empty = full + STAGES;
+    uint64_t *sf_ready = empty + STAGES;                                           // leader's are used
+    uint64_t *sf_empty = sf_ready + SLOTS;
+    uint64_t *tmem_full = sf_empty + SLOTS;
+    uint64_t *tmem_empty = tmem_full + 2;                                          // leader's are used
+    uint64_t *drain = tmem_empty + 2;
+    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 1);
+    volatile int *abort = reinterpret_cast<volatile int *>(tmem_base_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = (int)cluster_ctarank();
+    const bool leader = rank == 0;
+    const int t_first = blockIdx.x / 2, t_step = gridDim.x / 2;
+    const int tiles_mp = (g.tiles_m + 1) / 2;
+    const int groups = (g.num_kb + C::GROUP_KB - 1) / C::GROUP_KB;   // scale groups per tile
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int s = 0; s < SLOTS; ++s) {
+            mbar_init(&sf_ready[s], 2);           // the slot's warp of each CTA
+            mbar_init(&sf_empty[s], 1);
+        }
+        for (int a = 0; a < 2; ++a) {
+            mbar_init(&tmem_full[a], 1);
+            mbar_init(&tmem_empty[a], 2 * 128);   // the epilogue threads of both CTAs
+        }
+        mbar_init(drain, 1);
+        *abort = 0;
+        fence_barrier_init();
+        prefetch_tmap(&tmap_a);
+        prefetch_tmap(&tmap_b);
+    }
+    if (warp == 1) tmem_alloc_pair(tmem_base_slot, C::TMEM_COLS);
+    tc_fence_before();
+    cluster_sync_all();   // both CTAs' barriers exist before any remote arrival
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_base_slot;
+
+    auto coords = [&](int t, int &tm, int &tn) {
+        int pm = 0;
+        tile_coords(t, tiles_mp, g.tiles_n, pm, tn);
+        tm = 2 * pm + rank;   // past the last tile (odd count): zero rows, no stores
+    };
+
+    if (warp == 0) {
+        // ---------------- TMA producer (this CTA's half of every stage) ----------------
+        if (elect_one()) {
+            int stage = 0;
+            uint32_t phase = 0;
+            uint32_t issued_phase[STAGES];
+            bool issued[STAGES];
+            for (int s = 0; s < STAGES; ++s) issued[s] = false, issued_phase[s] = 0;
+            bool ok = true;
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
+                int tm, tn;
+                coords(t, tm, tn);
+                for (int kb = 0; kb < g.num_kb; kb += C::STAGE_KB) {
+                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, abort)) { ok = false; break; }
+                    const int steps = min(C::STAGE_KB, g.num_kb - kb);
+                    uint8_t *st = tiles + stage * C::STAGE_BYTES;
+                    const uint32_t fb = cluster_addr(&full[stage], 0);
+                    // both CTAs' loads land on the leader's barrier
+                    if (leader) mbar_expect_tx(&full[stage], 2u * (uint32_t)(steps * C::STEP_BYTES));
+#pragma unroll
+                    for (int q = 0; q < C::STAGE_KB; ++q) {
+                        if (q >= steps) break;
+                        const int blk = (kb + q) / g.kb_per_blk;
+                        const int kz = g.kept.idx[blk] * g.b + (kb + q - blk * g.kb_per_blk) * C::BKE;
+                        tma_load_2d_pair(&tmap_a, fb, st + q * C::STEP_BYTES, kz, tm * BM);
+                        tma_load_2d_pair(&tmap_b, fb, st + q * C::STEP_BYTES + C::A_BYTES, kz, tn * BN + rank * (BN / 2));
+                    }
+                    issued[stage] = true;
+                    issued_phase[stage] = phase;
+                    if (++stage == STAGES) stage = 0, phase ^= 1u;
+                }
+            }
+            // every stage this CTA loaded has been consumed by the pair's MMAs (so its
+            // copies have landed and no commit is still on its way here)
+            for (int s = 0; ok && s < STAGES; ++s)
+                if (issued[s] && !mbar_wait_cluster(&empty[s], issued_phase[s], abort)) ok = false;
+        }
+    } else if (warp == 1) {
+        // ---------------- MMA issuer (leader; one lane issues, the warp waits together) ----------------
+        if (leader) {
+            int stage = 0, slot = 0;
+            uint32_t phase = 0, sphase = 0;
+            int iter = 0;
+            bool ok = true;
+            bool any = false;
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step, ++iter) {
+                const int a = iter & 1;
+                const uint32_t aphase = (uint32_t)(iter >> 1) & 1u;
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, abort))) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem_base + (uint32_t)(a * 256);
+                for (int kb = 0; kb < g.num_kb; kb += C::STAGE_KB) {
+                    const uint32_t sfa = tmem_base + C::sfa(slot), sfb = sfa + 4;
+                    if (kb % C::GROUP_KB == 0) {
+                        if (!__all_sync(0xffffffffu, mbar_wait_cluster(&sf_ready[slot], sphase, abort))) { ok = false; break; }
+                        tc_fence_after();
+                        if (elect_one()) {
+                            const uint32_t ch = smem_u32(chunks + slot * C::CHUNKS * 512);
+#pragma unroll
+                            for (int c = 0; c < C::CHUNKS; ++c)
+                                tmem_cp_32x128b_x4_pair(sfa + 4 * c, sdesc_rows16(ch + 512 * c));
+                        }
+                        __syncwarp();
+                        any = true;
+                    }
+                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort))) { ok = false; break; }
+                    tc_fence_after();
+                    const int next = kb + C::STAGE_KB;
+                    const bool last = next % C::GROUP_KB == 0 || next >= g.num_kb;   // of the scale group
+                    if (elect_one()) {
+                        const uint32_t st = smem_u32(tiles + stage * C::STAGE_BYTES);
+#pragma unroll
+                        for (int q = 0; q < C::STAGE_KB; ++q) {
+                            if (kb + q >= g.num_kb) break;
+                            const uint32_t sa0 = st + q * C::STEP_BYTES, sb0 = sa0 + C::A_BYTES;
+                            const uint32_t byte = (uint32_t)((kb + q) % C::GROUP_KB);   // of the scale words
+                            const uint32_t idesc = C::IDESC | byte << 4 | byte << 29;
+#pragma unroll
+                            for (int kk = 0; kk < ROWB / 32; ++kk)
+                                umma_mxf8_pair(d, sdesc_kmajor_sw128(sa0 + kk * 32), sdesc_kmajor_sw128(sb0 + kk * 32),
+                                               idesc, sfa, sfb, (kb + q > 0 || kk > 0) ? 1u : 0u);
+                        }
+                        umma_commit_pair(&empty[stage], 0x3);   // the stage is free in both CTAs
+                        if (last) umma_commit_pair(&sf_empty[slot], 0x3);
+                    }
+                    __syncwarp();
+                    if (last && ++slot == SLOTS) slot = 0, sphase ^= 1u;
+                    if (++stage == STAGES) stage = 0, phase ^= 1u;
+                }
+                if (!ok) break;
+                if (elect_one()) umma_commit_pair(&tmem_full[a], 0x3);   // both halves of the accumulator
+                __syncwarp();
+            }
+            if (!ok && any && elect_one()) {
+                // drain: wait for the MMAs already issued before TMEM is freed
+                umma_commit_pair(drain, 0x1);
+                mbar_wait_drain(drain, 0);
+            }
+        }
+    } else if (warp >= 6) {
+        // ---------------- scales: warp 6 + s serves slot s in every round ----------------
+        const int slot = warp - 6;
+        uint32_t phase = 0;
+        const int64_t my_tiles = (g.num_tiles - t_first + t_step - 1) / t_step;
+        const int64_t total = my_tiles * groups;
+        uint8_t *ch = chunks + slot * C::CHUNKS * 512;
+        const uint32_t ready = cluster_addr(&sf_ready[slot], 0);
+        bool ok = true;
+        int64_t it = slot;
+        for (; it < total; it += SLOTS, phase ^= 1u) {
+            const int64_t ord = it / groups;
+            const int kb0 = (int)(it - ord * groups) * C::GROUP_KB;
+            int tm, tn;
+            coords(t_first + (int)ord * t_step, tm, tn);
+            uint32_t w[4 * C::CHUNKS];   // the words of rows lane + 32 u: A, then B
+#pragma unroll
+            for (int u = 0; u < 4 * C::CHUNKS; ++u) w[u] = 0;
+#pragma unroll
+            for (int q = 0; q < C::GROUP_KB; ++q) {
+                const int kb = min(kb0 + q, g.num_kb - 1);       // past the last step: any value
+                const int blk = kb / g.kb_per_blk;
+                const int64_t slice = (int64_t)g.kept.idx[blk] * g.kb_per_blk + (kb - blk * g.kb_per_blk);
+                const float *ra = sa + slice * ldsa, *rb = sb + slice * ldsb;
+#pragma unroll
+                for (int u = 0; u < 4 * C::CHUNKS; ++u) {
+                    const int64_t r = u < 4 ? (int64_t)tm * BM + 32 * u + lane : (int64_t)tn * BN + 32 * (u - 4) + lane;
+                    const bool in = u < 4 ? r < g.m : 32 * (u - 4) < BN && r < g.l;
+                    const float f = in ? __ldg((u < 4 ? ra : rb) + r) : 1.f;
+                    w[u] |= (ue8m0_x4(f) & 0xffu) << (8 * q);
+                }
+            }
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&sf_empty[slot], phase ^ 1u, abort))) { ok = false; break; }
+#pragma unroll
+            for (int c = 0; c < C::CHUNKS; ++c)
+                *reinterpret_cast<uint4 *>(ch + 512 * c + 16 * lane) =
+                    make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+            fence_proxy_async_smem();   // generic-proxy writes -> tcgen05.cp reads
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(ready);
+        }
+        // the last group of this slot has been consumed: no commit is still on its way here
+        if (ok && it > slot) mbar_wait_cluster(&sf_empty[slot], phase ^ 1u, abort);
+    } else {
+        // ---------------- epilogue (warps 2..5): this CTA's 128 rows ----------------
+        const int quarter = warp & 3;
+        float *buf = reinterpret_cast<float *>(chunks + SLOTS * C::CHUNKS * 512 + 256) + quarter * 32 * kEpiPitch;
+        const uint32_t empty_cl0 = cluster_addr(&tmem_empty[0], 0);
+        const uint32_t empty_cl1 = cluster_addr(&tmem_empty[1], 0);
+        const bool vec_ok = ((reinterpret_cast<uintptr_t>(g.C) & 15u) == 0) && (g.ldc % 4 == 0);
+        int iter = 0;
+        for (int t = t_first; t < g.num_tiles; t += t_step, ++iter) {
+            int tm, tn;
+            coords(t, tm, tn);
+            const int a = iter & 1;
+            const uint32_t aphase = (uint32_t)(iter >> 1) & 1u;
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, abort))) break;
+            tc_fence_after();
+            const int64_t r0 = (int64_t)tm * BM + quarter * 32, c0 = (int64_t)tn * BN;
+            for (int ch = 0; ch < BN / 32; ++ch) {
+                uint32_t v[32];
+                tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * 256 + ch * 32), v);
+                store_piece(buf, reinterpret_cast<const float *>(v), g.alpha, g.beta, g.C, g.ldc, r0, g.m, c0 + ch * 32,
+                            g.l, vec_ok, lane);
+            }
+            tc_fence_before();
+            mbar_arrive_cluster(a == 0 ? empty_cl0 : empty_cl1);
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync_all();   // both CTAs are done with the shared TMEM and with each other's barriers
+    if (warp == 1) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem_base, C::TMEM_COLS);
+    }
+}
+
 // ---------------------------------------------------------------- host ----
 
 typedef CUresult (*PFN_encodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
@@ -1528,6 +1806,55 @@ os_status launch_bf16(const void *A, int64_t lda, const void *B, int64_t ldb, in
     return launch_pair_bf16(A, lda, B, ldb, m, l, zK, blk, kept, alpha, beta, C, ldc, st);
 }
 
+// FP8 products: CTA pairs, or the one-CTA kernel when its tiles are few enough to share
+// K among a cluster or its waves cost less: on GB300 one takes 2.05 us + 0.418 per K step
+// of 128, one of tile pairs 3.1 us + 0.288 (equal at K = 1024).  GEMM, one CTA -> pairs, us:
+// 8192 x 8192 x 8192 465 -> 350, 3000 x 3000 x 4096 49.2 -> 38.9, 1500 x 1500 x 2048 16.3 ->
+// 14.6, 12288 x 300 x 8192 64.4 -> 51.3; and where the one-CTA kernel stays: 1300 x 12288 x
+// 1024 26.9 -> 32.9, 4096 x 4096 x 512 24.7 -> 26.2, 1000 x 700 x 2048 (split) 12.3 -> 14.4.
+os_status launch_fp8(const void *A, const float *sa, int64_t lda, const void *B, const float *sb, int64_t ldb, int64_t m,
+                     int64_t l, int64_t zK, int32_t blk, const BlockList &kept, float alpha, float beta, float *Cout,
+                     int64_t ldc, cudaStream_t st) {
+    using C = CfgPairFp8;
+    const int kb = (int)(kept.count * (int64_t)blk / C::BKE);
+    const int64_t ones = (m + BM - 1) / BM * ((l + CfgFp8::BN - 1) / CfgFp8::BN);
+    const int64_t pairs = (m + 2 * BM - 1) / (2 * BM) * ((l + C::BN - 1) / C::BN);
+    auto waves = [](int64_t tiles, int64_t at_once) { return (double)((tiles + at_once - 1) / at_once); };
+    if (split_of<CfgFp8>(ones, kb, CfgFp8::MIN_SPLIT_KB) > 1 ||
+        waves(ones, num_sms()) * (2.05 + 0.418 * kb) <= waves(pairs, num_sms() / 2) * (3.1 + 0.288 * kb))
+        return launch_tc<CfgFp8>(A, sa, lda, B, sb, ldb, m, l, zK, blk, kept, alpha, beta, Cout, ldc, st);
+    if (blk % C::BKE != 0 || zK >= (int64_t(1) << 31)) return OS_ERR_UNSUPPORTED;
+    if (!aligned16(A) || !aligned16(B) || lda % 16 != 0 || ldb % 16 != 0 || !aligned16(sa) || !aligned16(sb))
+        return OS_ERR_INVALID_ARG;
+    GemmArgs g;
+    std::memset(&g, 0, sizeof(g));
+    g.m = m;
+    g.l = l;
+    g.b = blk;
+    g.kb_per_blk = blk / C::BKE;
+    g.kept = kept;
+    g.num_kb = kept.count * g.kb_per_blk;
+    g.tiles_m = (int)((m + BM - 1) / BM);
+    g.tiles_n = (int)((l + C::BN - 1) / C::BN);
+    g.num_tiles = (g.tiles_m + 1) / 2 * g.tiles_n;   // tile pairs
+    g.alpha = alpha;
+    g.beta = beta;
+    g.C = Cout;
+    g.ldc = ldc;
+    CUtensorMap ta, tb;
+    OSK_TRY(make_tmap(&ta, A, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, m, zK, lda, BM, C::BKE));
+    OSK_TRY(make_tmap(&tb, B, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, l, zK, ldb, C::BN / 2, C::BKE));
+    static std::once_flag attr_once;
+    static cudaError_t attr_err = cudaSuccess;
+    std::call_once(attr_once, [] {
+        attr_err = cudaFuncSetAttribute(gemm_pair_fp8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    });
+    OSK_CUDA_TRY(attr_err);
+    OSK_CUDA_TRY(launch_pairs(gemm_pair_fp8_kernel, C::THREADS, C::SMEM, g.num_tiles, st, ta, tb, sa,
+                              (int64_t)fp8_scale_ld(m), sb, (int64_t)fp8_scale_ld(l), g));
+    return check_launch();
+}
+
 }  // namespace
 
 // The backward pass's products straight from the sketched operands: T = dC
@@ -1616,8 +1943,7 @@ os_status gemm_masked_tc(const Plan *p, const void *At, int64_t ldat, const floa
     }
     if (dt == OS_FP8E4M3) {
         if (!a_scales || !b_scales) return OS_ERR_INVALID_ARG;
-        return launch_tc<CfgFp8>(At, a_scales, ldat, BtT, b_scales, ldbt, m, l, z, p->b, kept, alpha, beta, C, ldc,
-                                 st);
+        return launch_fp8(At, a_scales, ldat, BtT, b_scales, ldbt, m, l, z, p->b, kept, alpha, beta, C, ldc, st);
     }
     return OS_ERR_UNSUPPORTED;
 }

@@ -321,7 +321,7 @@ def run_ours(args):
                           max(ops.sketch_workspace(p, w.m), ops.sketch_workspace(p, w.l)), dtype=torch.uint8, device=dev)
     stream = torch.cuda.current_stream()
 
-    # the same three calls oversketch_matmul makes: only kept blocks are sketched
+    # the three calls of oversketch_matmul (f32: its 3xTF32 form): only kept blocks are sketched
     def step():
         ops.sketch_left(p, A, sd, out=At, scales=a_sc, workspace=ws_pack, block_mask=w.mask)
         ops.sketch_right(p, B, sd, out=BtT, scales=b_sc, block_mask=w.mask, workspace=ws_pack)
@@ -461,7 +461,7 @@ def run_ours(args):
             peak = peaks.get("bf16_tflops", peaks.get("bf16_tflops_sustained"))
         elif sd == "fp8":
             # block-scaled E4M3: nominal FP8 : BF16 tensor rate = 2 : 1
-            dom = "gemm_masked_tc_kernel<Cfg<224,4,Fp8>> (E4M3, UE8M0 block scales)"
+            dom = "gemm_pair_fp8_kernel (E4M3, UE8M0 block scales, cta_group::2)"
             peak = 2.0 * peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
         elif sd == "tf32x2":
             # three TF32 products per K step at half the BF16 rate: the useful FP32 rate peaks

@@ -13,7 +13,7 @@
 // The gather reads X in strips of W free indices (W = 128 for FP32, 256 for
 // BF16): strip s holds X[0..n-1, Ws .. Ws+W-1], and a random row of it is one
 // 512-byte piece, 16 bytes per lane of a warp.  The left operand (and a BF16
-// right operand) is first packed strip-major into the workspace, n contiguous
+// right operand whose rows are not 16-byte aligned) is first packed strip-major into the workspace, n contiguous
 // rows of 128 elements per strip, zero-padded past the free extent; packing
 // the left operand is the transpose it needs anyway.  An FP32 right operand
 // is gathered in place: in 128-wide strips when its rows are 16-byte aligned,
@@ -45,7 +45,6 @@ namespace osk {
 
 namespace {
 
-constexpr int kTileQ = 128;
 constexpr int kWarps = 8;
 constexpr int kStrip = 128;   // free indices per FP32 strip (the in-place right sketch)
 
@@ -55,7 +54,6 @@ template <typename T>
 __host__ __device__ constexpr int strip_of() {
     return 32 * (16 / (int)sizeof(T));
 }
-constexpr int kUnroll = 8;
 
 // VW consecutive elements of the free dimension per lane (strip = 32*VW).
 template <typename InT, int VW, bool kAligned>

@@ -30,7 +30,7 @@ os_status gemm_masked_f32(const Plan *p, const float *At, int64_t ldat, const fl
 os_status unsketch_cols_t_impl(const Plan *p, const float *Tt, int64_t m, int64_t ldt, uint64_t mask, void *dX,
                                os_dtype x_t, int64_t ldx, cudaStream_t st);
 os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &b, int64_t ld, int64_t l,
-                            uint64_t mask, float alpha, float *C, int64_t ldc, unsigned int *flag, cudaStream_t st);
+                            uint64_t mask, float alpha, float *C, int64_t ldc, SplitCtl *ctl, cudaStream_t st);
 os_status gemm_bf16_mn(const void *A, int64_t lda, bool a_mn, const void *B, int64_t ldb, bool b_mn, int64_t m,
                        int64_t l, int64_t K, float alpha, float *C, int64_t ldc, int32_t mn_b, int32_t remap,
                        uint64_t mask, int32_t P, cudaStream_t st);
@@ -115,7 +115,7 @@ MatmulLayout layout(const Plan *p, int64_t m, int64_t l, os_dtype a_t, os_dtype 
 
 // Whether an FP32 product runs on FP16 planes (sketches as FP32 sums, split row by
 // row, gemm_masked_f16x3) instead of on TF32 planes written by the sketches: block
-// widths that fit the 64-element K tile, scratch space for the row scales, and a
+// widths that fit the 64-element K tile, scratch space for what the split leaves, and a
 // GEMM that gains more than the split and its launches cost.  On GB300 a 128 x 128
 // tile of the 3xTF32 kernel takes 19.5 ns per K (152 at once, K shared by up to eight
 // CTAs when there are few tiles: tf32x3_us), a 256 x 160 tile of the FP16 one 10.2 ns
@@ -127,7 +127,7 @@ MatmulLayout layout(const Plan *p, int64_t m, int64_t l, os_dtype a_t, os_dtype 
 // 342 -> 348.
 bool f16x3_pays(const Plan *p, os_dtype gemm_dtype, int64_t m, int64_t l, uint64_t mask, size_t scratch) {
     if (gemm_dtype != OS_F32 || p->b % 64 != 0) return false;
-    if (scratch < (size_t)(m + l) * 4 + 512) return false;
+    if (scratch < (size_t)(m + l) * 4 + sizeof(SplitCtl) + 256) return false;
     const double K = (double)__builtin_popcountll(mask) * p->b;
     auto waves = [](int64_t tiles, int at_once) { return (double)((tiles + at_once - 1) / at_once); };
     const double tf32 = tf32x3_us(m, l, (int64_t)K);
@@ -136,14 +136,14 @@ bool f16x3_pays(const Plan *p, os_dtype gemm_dtype, int64_t m, int64_t l, uint64
 }
 
 // The masked product of FP32 sums stored as TF32 pairs are (sums, then a plane's
-// room), by f16x3_pays; scratch holds the row scales and the flag.
+// room), by f16x3_pays; scratch holds the split's control words and the row scales.
 os_status matmul_f16x3(const Plan *p, void *At, void *BtT, int64_t ld, int64_t m, int64_t l, uint64_t mask, float *C,
                        int64_t ldc, void *scratch, cudaStream_t st) {
-    unsigned int *flag = reinterpret_cast<unsigned int *>((reinterpret_cast<uintptr_t>(scratch) + 255) & ~uintptr_t(255));
-    float *sa = reinterpret_cast<float *>(flag + 4);
+    SplitCtl *ctl = reinterpret_cast<SplitCtl *>((reinterpret_cast<uintptr_t>(scratch) + 255) & ~uintptr_t(255));
+    float *sa = reinterpret_cast<float *>(ctl + 1);
     const SplitSide a{reinterpret_cast<float *>(At), m, sa};
     const SplitSide b{reinterpret_cast<float *>(BtT), BtT == At ? 0 : l, BtT == At ? sa : sa + m};
-    return gemm_masked_f16x3(p, a, b, ld, l, mask, 1.0f / (float)__builtin_popcountll(mask), C, ldc, flag, st);
+    return gemm_masked_f16x3(p, a, b, ld, l, mask, 1.0f / (float)__builtin_popcountll(mask), C, ldc, ctl, st);
 }
 
 // Deterministic FP64 partial sums: fixed grid, fixed per-thread order, fixed tree.

@@ -53,6 +53,16 @@ struct SplitSide {
     float *scale;
 };
 
+// What the split leaves for the launches after it, in the product's scratch: flag, set
+// when the planes do not suit the operands (the product then runs on TF32 planes), and
+// the entries left out of the planes: their count, then row (bit 31: of B) and column.
+// 2048 entries: operands of random sums have a few, heavy-tailed ones some hundred.
+constexpr unsigned int kSplitLost = 2048;
+struct SplitCtl {
+    unsigned int flag, lost, pad[2];
+    uint2 entry[kSplitLost];
+};
+
 os_status set_cuda_error(cudaError_t err);
 os_status check_launch();
 BlockList mask_to_list(uint64_t mask, int P);

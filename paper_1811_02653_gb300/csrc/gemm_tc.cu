@@ -38,9 +38,9 @@ namespace osk {
 
 // implemented in split.cu
 os_status launch_split_f16(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
-                           unsigned int *flag, cudaStream_t st);
-os_status launch_tf32_planes(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
-                             const unsigned int *flag, cudaStream_t st);
+                           SplitCtl *ctl, cudaStream_t st);
+os_status launch_split_correct(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
+                               const SplitCtl *ctl, float alpha, float *C, int64_t ldc, int64_t l, cudaStream_t st);
 
 namespace {
 
@@ -950,7 +950,7 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
 
 // ---------------------------------------------------------------------------
 // FP32-accuracy masked GEMM on FP16 planes (split.cu), CTA pairs:
-//   A~ B~ = hi.hi + (hi.lo + lo.hi) / 2048        (lo.lo, 2^-24 of the terms, dropped)
+//   A~ B~ = hi.hi + (hi.lo + lo.hi) / 2048        (lo.lo, up to 2^-22 of the terms, dropped)
 // The organisation of gemm_pair_bf16_kernel with 256 x 160 tiles and two kinds of
 // accumulators: hi.hi in chunks of K = 256, double-buffered, which the epilogue
 // adds in FP32 registers (the tensor core's FP32 accumulation truncates, so its
@@ -1868,18 +1868,18 @@ os_status gemm_bf16_mn(const void *A, int64_t lda, bool a_mn, const void *B, int
 }
 
 // The FP32-accuracy product from FP32 sums on FP16 planes (gemm_pair_f16x3_kernel):
-// split both operands, multiply, and behind the split's flag the 3xTF32 product of
-// the same sums for operands that the planes do not suit.  B's rows = 0: B is A.
+// split both operands, multiply, add the products of the entries that the split left out
+// of the planes, and behind the split's flag the 3xTF32 product of the same sums for
+// operands that the planes do not suit.  B's rows = 0: B is A.
 os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &b, int64_t ld, int64_t l,
-                            uint64_t mask, float alpha, float *Cout, int64_t ldc, unsigned int *flag,
-                            cudaStream_t st) {
+                            uint64_t mask, float alpha, float *Cout, int64_t ldc, SplitCtl *ctl, cudaStream_t st) {
     using C = CfgF16x3;
     const BlockList kept = mask_to_list(mask, p->P);
     const SplitSide &bs = b.rows ? b : a;
     const int64_t m = a.rows, z = (int64_t)p->P * p->b;
     if (p->b % C::BKE != 0 || z >= (int64_t(1) << 31)) return OS_ERR_UNSUPPORTED;
     if (!aligned16(a.sums) || !aligned16(bs.sums) || ld % 8 != 0) return OS_ERR_INVALID_ARG;
-    OSK_TRY(launch_split_f16(a, b, ld, p->b, kept, flag, st));
+    OSK_TRY(launch_split_f16(a, b, ld, p->b, kept, ctl, st));
     GemmArgs g;
     std::memset(&g, 0, sizeof(g));
     g.m = m;
@@ -1896,7 +1896,7 @@ os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &
     g.ldc = ldc;
     g.a_scale = a.scale;
     g.b_scale = bs.scale;
-    g.skip_if = flag;
+    g.skip_if = &ctl->flag;
     const uint16_t *ah = reinterpret_cast<const uint16_t *>(a.sums + m * ld);
     const uint16_t *bh = reinterpret_cast<const uint16_t *>(bs.sums + bs.rows * ld);
     CUtensorMap tah, tal, tbh, tbl;
@@ -1914,9 +1914,9 @@ os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &
     OSK_CUDA_TRY(attr_err);
     OSK_CUDA_TRY(launch_pairs(gemm_pair_f16x3_kernel, C::THREADS, C::SMEM, g.num_tiles, st, tah, tal, tbh, tbl, g));
     OSK_TRY(check_launch());
-    OSK_TRY(launch_tf32_planes(a, b, ld, p->b, kept, flag, st));
+    OSK_TRY(launch_split_correct(a, b, ld, p->b, kept, ctl, alpha, Cout, ldc, l, st));
     return launch_tc<CfgTf32x3>(a.sums, a.sums + m * ld, ld, bs.sums, bs.sums + bs.rows * ld, ld, m, l, z, p->b, kept,
-                                alpha, 0.f, Cout, ldc, st, flag);
+                                alpha, 0.f, Cout, ldc, st, &ctl->flag);
 }
 
 // The 3xTF32 kernel's time for a product by its tiles and their split, in us (19.5 ns

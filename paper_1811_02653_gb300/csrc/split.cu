@@ -3,16 +3,21 @@
 // A row of FP32 sums x is written as hi + lo / 2048 with hi and lo in FP16 after a
 // power-of-two scale 2^-e that brings the row's largest magnitude into [2^14, 2^15):
 //   hi = RN16(x 2^-e),   lo = RN16((x 2^-e - hi) 2048)      (the difference is exact)
-// so x 2^-e = hi + lo / 2048 to 2^-24 of x for every |x| >= 2^-28 of the row's
-// largest (below that, to 2^-36 of the scale's unit).  3xTF32 keeps 22 bits of x
-// (both of its planes lose bits by truncation), and the FP16 tensor rate is twice
-// the TF32 one.
+// so hi + lo / 2048 is x 2^-e to 2^-23 of it wherever |x 2^-e| >= 2^-13 (hi leaves at
+// most 2^-11, of which lo keeps 11 bits), that is down to 2^-28 of the row's largest.
+// 3xTF32 holds x to 2^-20 (its planes keep 11 bits each by truncation), and the FP16
+// tensor rate is twice the TF32 one.
 //
-// Rows that the format does not suit are counted on the device: a largest magnitude
-// that is not finite or lies outside [2^-40, 2^60], or more than a 64th of the
-// nonzeros below 2^-28 of the largest.  One such row raises *flag; the FP16 product
-// then returns at once and the TF32 planes are made from the same sums in place
-// (tf32_planes_kernel), so that these operands keep the accuracy they had.
+// Below 2^-13 FP16 runs out of exponents: the planes would be off by up to 2^-36, any
+// share of x, and more of x in lo makes more of the dropped lo.lo.  How few such entries
+// a row has says nothing about what they contribute (C consists of them where the other
+// operand is zero beside them), so none is left to the planes: they get zeros there, the
+// entries are listed, and correct_kernel adds their products to C in FP32.  Sums of
+// random signs have some by chance (two or three in the 2^27 sums of an 8192 x 32768 x
+// 8192 product); operands with more than the list holds (columns of very different
+// scale, say) raise the flag, and so does a row whose largest magnitude is not finite or
+// lies outside [2^-40, 2^60].  The FP16 product then returns at once and the TF32 planes
+// are made from the same sums in place, so these operands get the 3xTF32 product.
 //
 // The split is memory-bound: 2 x 8192 rows of 8192 sums, 4 bytes read (twice, the
 // second time from L1/L2) and 4 written each, take 165 us (6.5 TB/s) on GB300.
@@ -26,9 +31,13 @@ namespace {
 
 constexpr uint32_t kAmaxLo = 0x2b800000u;   // 2^-40
 constexpr uint32_t kAmaxHi = 0x5d800000u;   // 2^60
+constexpr float kExactFrom = 0x1p-13f;      // scaled magnitudes from here on are held to 2^-23
+
+// Whether a scaled sum is left to the list.
+__device__ __forceinline__ bool listed(float v) { return v != 0.f && fabsf(v) < kExactFrom; }
 
 __global__ void __launch_bounds__(256) split_f16_kernel(SplitSide a, SplitSide b, int64_t ld, int32_t blk,
-                                                        BlockList kept, unsigned int *__restrict__ flag) {
+                                                        BlockList kept, SplitCtl *__restrict__ ctl) {
     const bool right = blockIdx.x >= (uint64_t)a.rows;
     const SplitSide s = right ? b : a;
     const int64_t r = right ? (int64_t)blockIdx.x - a.rows : (int64_t)blockIdx.x;
@@ -38,7 +47,8 @@ __global__ void __launch_bounds__(256) split_f16_kernel(SplitSide a, SplitSide b
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int per = blk / 4, total = kept.count * per;   // 16-byte pieces
     __shared__ uint32_t red[8];
-    __shared__ int2 cnt[8];
+    __shared__ int cnt[8];
+    __shared__ unsigned int at;
     auto piece = [&](int q) -> int64_t {
         const int t = q / per;
         return (int64_t)kept.idx[t] * blk + 4 * (q - t * per);
@@ -48,7 +58,8 @@ __global__ void __launch_bounds__(256) split_f16_kernel(SplitSide a, SplitSide b
 #pragma unroll 4
     for (int q = tid; q < total; q += 256) {
         const uint4 u = *reinterpret_cast<const uint4 *>(x + piece(q));
-        am = max(max(am, u.x & 0x7fffffffu), max(u.y & 0x7fffffffu, max(u.z & 0x7fffffffu, u.w & 0x7fffffffu)));
+        am = max(am, max(u.x & 0x7fffffffu, u.y & 0x7fffffffu));
+        am = max(am, max(u.z & 0x7fffffffu, u.w & 0x7fffffffu));
     }
     am = __reduce_max_sync(0xffffffffu, am);
     if (lane == 0) red[warp] = am;
@@ -56,12 +67,12 @@ __global__ void __launch_bounds__(256) split_f16_kernel(SplitSide a, SplitSide b
 #pragma unroll
     for (int w = 0; w < 8; ++w) am = max(am, red[w]);
     if (am != 0 && (am < kAmaxLo || am > kAmaxHi)) {
-        if (tid == 0) *flag = 1u;
+        if (tid == 0) ctl->flag = 1u;
         return;
     }
     const int e = am ? (int)(am >> 23) - 127 - 14 : 0;
     const float down = __uint_as_float((uint32_t)(127 - e) << 23);   // 2^-e, exact
-    int nz = 0, small = 0;
+    int small = 0;
 #pragma unroll 4
     for (int q = tid; q < total; q += 256) {
         const int64_t c = piece(q);
@@ -70,60 +81,131 @@ __global__ void __launch_bounds__(256) split_f16_kernel(SplitSide a, SplitSide b
         __half h[4], l[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            h[k] = __float2half_rn(v[k]);
-            l[k] = __float2half_rn((v[k] - __half2float(h[k])) * 2048.f);
-            nz += v[k] != 0.f;
-            small += v[k] != 0.f && fabsf(v[k]) < 0x1p-13f;
+            const float p = fabsf(v[k]) < kExactFrom ? 0.f : v[k];
+            h[k] = __float2half_rn(p);
+            l[k] = __float2half_rn((p - __half2float(h[k])) * 2048.f);
+            small += p != v[k];
         }
         *reinterpret_cast<uint2 *>(hi + c) = *reinterpret_cast<const uint2 *>(h);
         *reinterpret_cast<uint2 *>(lo + c) = *reinterpret_cast<const uint2 *>(l);
     }
-    nz = __reduce_add_sync(0xffffffffu, nz);
+    if (tid == 0) s.scale[r] = __uint_as_float((uint32_t)(127 + e) << 23);   // 2^e
     small = __reduce_add_sync(0xffffffffu, small);
-    if (lane == 0) cnt[warp] = make_int2(nz, small);
+    if (lane == 0) cnt[warp] = small;
     __syncthreads();
+    int n = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) n += cnt[w];
+    if (n == 0) return;
+    // the row's entries for the list: consecutive, by ascending column
     if (tid == 0) {
-        int n = 0, t = 0;
-        for (int w = 0; w < 8; ++w) n += cnt[w].x, t += cnt[w].y;
-        if ((int64_t)t * 64 > n) *flag = 1u;
-        s.scale[r] = __uint_as_float((uint32_t)(127 + e) << 23);   // 2^e
+        at = n <= kSplitLost ? atomicAdd(&ctl->lost, (unsigned int)n) : kSplitLost;
+        if (at + n > kSplitLost) ctl->flag = 1u;
+    }
+    __syncthreads();
+    unsigned int base = at;
+    if (base + n > kSplitLost) return;
+    for (int q0 = 0; q0 < total; q0 += 256) {
+        const int q = q0 + tid;
+        const int64_t c = q < total ? piece(q) : 0;
+        const float4 u = q < total ? *reinterpret_cast<const float4 *>(x + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float v[4] = {u.x * down, u.y * down, u.z * down, u.w * down};
+        int mine = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) mine += listed(v[k]);
+        int inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        __syncthreads();   // cnt has been read
+        if (lane == 31) cnt[warp] = inc;
+        __syncthreads();
+        unsigned int pos = base + inc - mine;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) pos += cnt[w];
+            base += cnt[w];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (listed(v[k])) ctl->entry[pos++] = make_uint2((uint32_t)r | (right ? 0x80000000u : 0u), (uint32_t)(c + k));
     }
 }
 
-// The sums as the two TF32 planes (hi in place, lo over the FP16 planes), when *flag is set.
-__global__ void __launch_bounds__(256) tf32_planes_kernel(SplitSide a, SplitSide b, int64_t ld, int32_t blk,
-                                                          BlockList kept, const unsigned int *__restrict__ flag) {
-    if (*flag == 0u) return;
-    const int per = blk / 4, total = kept.count * per;
-    for (int64_t row = blockIdx.x; row < a.rows + b.rows; row += gridDim.x) {
-        const SplitSide &s = row < a.rows ? a : b;
-        float *x = s.sums + (row < a.rows ? row : row - a.rows) * ld;
-        float *y = x + s.rows * ld;
-        for (int q = threadIdx.x; q < total; q += 256) {
-            const int t = q / per;
-            const int64_t c = (int64_t)kept.idx[t] * blk + 4 * (q - t * per);
-            const float4 u = *reinterpret_cast<const float4 *>(x + c);
-            auto top = [](float v) { return __uint_as_float(__float_as_uint(v) & 0xffffe000u); };
-            const float4 h = make_float4(top(u.x), top(u.y), top(u.z), top(u.w));
-            *reinterpret_cast<float4 *>(x + c) = h;
-            *reinterpret_cast<float4 *>(y + c) = make_float4(u.x - h.x, u.y - h.y, u.z - h.z, u.w - h.w);
+// After the FP16 product: with the flag set, the sums as the two TF32 planes (hi in
+// place, lo over the FP16 planes) for the 3xTF32 product that follows; else the products
+// of the listed entries, added to C: those of A with all of B, those of B with what the
+// planes hold of A.  Tiles of 256 x 256 of C, one owner each: first the entries of A in
+// its rows (thread = column), then those of B in its columns (thread = row).  The entries
+// of one row are consecutive and ascending in the list and no two rows meet in an
+// element, so the sums do not depend on the order in which the rows entered it.  Nothing
+// listed: two loads.
+__global__ void __launch_bounds__(256) correct_kernel(SplitSide a, SplitSide b, int64_t ld, int32_t blk,
+                                                      BlockList kept, const SplitCtl *__restrict__ ctl, float alpha,
+                                                      float *__restrict__ C, int64_t ldc, int64_t l) {
+    if (ctl->flag != 0u) {
+        const int per = blk / 4, total = kept.count * per;
+        for (int64_t row = blockIdx.x; row < a.rows + b.rows; row += gridDim.x) {
+            const SplitSide &s = row < a.rows ? a : b;
+            float *x = s.sums + (row < a.rows ? row : row - a.rows) * ld;
+            float *y = x + s.rows * ld;
+            for (int q = threadIdx.x; q < total; q += 256) {
+                const int t = q / per;
+                const int64_t c = (int64_t)kept.idx[t] * blk + 4 * (q - t * per);
+                const float4 u = *reinterpret_cast<const float4 *>(x + c);
+                auto top = [](float v) { return __uint_as_float(__float_as_uint(v) & 0xffffe000u); };
+                const float4 h = make_float4(top(u.x), top(u.y), top(u.z), top(u.w));
+                *reinterpret_cast<float4 *>(x + c) = h;
+                *reinterpret_cast<float4 *>(y + c) = make_float4(u.x - h.x, u.y - h.y, u.z - h.z, u.w - h.w);
+            }
         }
+        return;
+    }
+    const int lost = (int)ctl->lost;
+    if (lost == 0) return;
+    __shared__ uint2 list[kSplitLost];
+    for (int i = threadIdx.x; i < lost; i += 256) list[i] = ctl->entry[i];
+    __syncthreads();
+    const bool sym = b.rows == 0;   // B is A: its entries count on both sides
+    const SplitSide &bs = sym ? a : b;
+    const int64_t tm = (a.rows + 255) / 256, tn = (l + 255) / 256;
+    for (int64_t t = blockIdx.x; t < tm * tn; t += gridDim.x) {
+        const int64_t r0 = t / tn * 256, s0 = (t - t / tn * tn) * 256;
+        const int64_t col = s0 + threadIdx.x, row = r0 + threadIdx.x;
+        for (int i = 0; i < lost; ++i) {
+            const int64_t r = list[i].x, c = list[i].y;
+            if ((list[i].x >> 31) || r < r0 || r >= r0 + 256 || col >= l) continue;
+            float *dst = C + r * ldc + col;
+            *dst = fmaf(alpha * a.sums[r * ld + c], bs.sums[col * ld + c], *dst);
+        }
+        __syncthreads();   // the rows above may hold elements of the columns below
+        for (int i = 0; i < lost; ++i) {
+            const int64_t s = list[i].x & 0x7fffffffu, c = list[i].y;
+            if ((sym ? 0u : 1u) != list[i].x >> 31 || s < s0 || s >= s0 + 256 || row >= a.rows) continue;
+            const float x = a.sums[row * ld + c];
+            if (listed(x * (1.f / a.scale[row]))) continue;   // added above
+            float *dst = C + row * ldc + s;
+            *dst = fmaf(alpha * x, bs.sums[s * ld + c], *dst);
+        }
+        __syncthreads();
     }
 }
 
 }  // namespace
 
 os_status launch_split_f16(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
-                           unsigned int *flag, cudaStream_t st) {
-    OSK_CUDA_TRY(cudaMemsetAsync(flag, 0, sizeof(unsigned int), st));
-    split_f16_kernel<<<(unsigned)(a.rows + b.rows), 256, 0, st>>>(a, b, ld, blk, kept, flag);
+                           SplitCtl *ctl, cudaStream_t st) {
+    OSK_CUDA_TRY(cudaMemsetAsync(ctl, 0, offsetof(SplitCtl, entry), st));
+    split_f16_kernel<<<(unsigned)(a.rows + b.rows), 256, 0, st>>>(a, b, ld, blk, kept, ctl);
     return check_launch();
 }
 
-os_status launch_tf32_planes(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
-                             const unsigned int *flag, cudaStream_t st) {
+os_status launch_split_correct(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
+                               const SplitCtl *ctl, float alpha, float *C, int64_t ldc, int64_t l, cudaStream_t st) {
     const int64_t rows = a.rows + b.rows;
-    tf32_planes_kernel<<<(unsigned)(rows < 152 * 8 ? rows : 152 * 8), 256, 0, st>>>(a, b, ld, blk, kept, flag);
+    correct_kernel<<<(unsigned)(rows < 152 * 8 ? rows : 152 * 8), 256, 0, st>>>(a, b, ld, blk, kept, ctl, alpha, C, ldc, l);
     return check_launch();
 }
 

@@ -16,7 +16,7 @@
 // random signs have some by chance (two or three in the 2^27 sums of an 8192 x 32768 x
 // 8192 product); operands with more than the list holds (columns of very different
 // scale, say) raise the flag, and so does a row whose largest magnitude is not finite or
-// lies outside [2^-40, 2^60].  The FP16 product then returns at once and the TF32 planes
+// lies outside [2^-60, 2^80].  The FP16 product then returns at once and the TF32 planes
 // are made from the same sums in place, so these operands get the 3xTF32 product.
 //
 // The split is memory-bound: 2 x 8192 rows of 8192 sums, 4 bytes read (twice, the
@@ -29,8 +29,10 @@ namespace osk {
 
 namespace {
 
-constexpr uint32_t kAmaxLo = 0x2b800000u;   // 2^-40
-constexpr uint32_t kAmaxHi = 0x5d800000u;   // 2^60
+// A row's largest magnitude: between these, a sum of products of scaled values (2^-50 ..
+// 2^48) times one side's scale stays a normal number before the other's is applied.
+constexpr uint32_t kAmaxLo = 0x21800000u;   // 2^-60
+constexpr uint32_t kAmaxHi = 0x67800000u;   // 2^80
 constexpr float kExactFrom = 0x1p-13f;      // scaled magnitudes from here on are held to 2^-23
 
 // Whether a scaled sum is left to the list.
@@ -53,6 +55,8 @@ __global__ void __launch_bounds__(256) split_f16_kernel(SplitSide a, SplitSide b
         const int t = q / per;
         return (int64_t)kept.idx[t] * blk + 4 * (q - t * per);
     };
+    // another row has raised the flag: nothing of this pass will be used
+    if (__syncthreads_or(tid == 0 && *(volatile unsigned int *)&ctl->flag != 0u)) return;
     // the row's largest magnitude (as bits: NaN above Inf above every finite value)
     uint32_t am = 0;
 #pragma unroll 4

@@ -433,13 +433,15 @@ OS_API os_status oversketch_frob(const float *X, int64_t ldx, const float *Y, in
 OS_API os_status oversketch_device_status(void *stream, int32_t *status, int32_t reset);
 
 /* Test hook of the bounded waits; the paper has no counterpart.  With
- * skip_kb >= 0, the next launch of the one-CTA tensor-core GEMM (the FP8 and
- * 3xTF32 masked products, grouped BF16 launches) leaves K step skip_kb of its
- * first CTA's first tile unloaded and unarmed, and gives that CTA a wait limit
- * of limit_ns (> 0) instead of one second: the MMA warp's wait for that stage
- * runs out, the CTA records OS_ERR_TIMEOUT, waits (one second at most) for the
- * copies it did issue, frees its tensor memory and returns.  The setting is
- * consumed by that one launch; skip_kb < 0 withdraws a pending one.
+ * skip_kb >= 0, the next launch of a tensor-core GEMM kernel (every masked,
+ * per-block, grouped, BF16 or backward product but the FFMA one; an FP32 product
+ * that goes back from FP16 to TF32 planes: the TF32 one) leaves K step skip_kb
+ * (the stage that holds it) of its first CTA's or CTA pair's first tile unloaded
+ * and unarmed, and gives that CTA or pair a wait limit of limit_ns (> 0) instead
+ * of one second: the MMA warp's wait for that stage runs out, the CTA records
+ * OS_ERR_TIMEOUT, waits (one second at most) for the copies it did issue, frees
+ * its tensor memory and returns.  The setting is consumed by that one launch,
+ * whether its first tile has that K step or not; skip_kb < 0 withdraws a pending one.
  * Synchronous (device-wide symbol copies).  Errors: OS_ERR_INVALID_ARG
  * (limit_ns == 0 with skip_kb >= 0), OS_ERR_CUDA. */
 OS_API os_status oversketch_test_wait_timeout(uint64_t limit_ns, int32_t skip_kb);

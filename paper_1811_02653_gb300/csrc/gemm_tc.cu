@@ -686,7 +686,8 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
 //   warp 0      TMA producer of this CTA's half (completion on the leader's barrier)
 //   warp 1      TMEM (both CTAs, jointly); MMA issue and commits (leader)
 //   warps 2..5  epilogue of this CTA's 128 rows; release the accumulator on the leader
-// Waits are bounded as in gemm_masked_tc_kernel.
+// Waits are bounded as in gemm_masked_tc_kernel; a producer that gives up drains its
+// CTA's copies by drain_pair_copies.
 struct CfgPair {
     static constexpr int BN = 256;                    // tile columns (the pair's N)
     static constexpr int STAGES = 6;
@@ -723,8 +724,8 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
     uint64_t *tmem_full = empty + STAGES;
     uint64_t *tmem_empty = tmem_full + 2;                                          // leader's are used
     uint64_t *drain = tmem_empty + 2;
-    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 1);
-    volatile int *abort = reinterpret_cast<volatile int *>(tmem_base_slot + 1);
+    volatile WaitState *wait = reinterpret_cast<volatile WaitState *>(drain + 1);
+    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 3);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)cluster_ctarank();
@@ -742,15 +743,16 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
             mbar_init(&tmem_empty[a], 2 * 128);   // the epilogue threads of both CTAs
         }
         mbar_init(drain, 1);
-        *abort = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap_a);
         prefetch_tmap(&tmap_b);
     }
+    if (threadIdx.x == 64) wait_state_init(wait);
     if (warp == 1) tmem_alloc_pair(tmem_base_slot, C::TMEM_COLS);
     tc_fence_before();
     cluster_sync_all();   // both CTAs' barriers exist before any remote arrival
     tc_fence_after();
+    if (threadIdx.x == 64) wait_state_taken(wait);
     const uint32_t tmem_base = *tmem_base_slot;
 
     auto coords = [&](int t, int &tm, int &tn) {
@@ -786,19 +788,22 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t issued_phase[STAGES];
-            bool issued[STAGES];
-            for (int s = 0; s < STAGES; ++s) issued[s] = false, issued_phase[s] = 0;
+            uint32_t issued = 0, issued_phase = 0;   // bit s: stage s was loaded, and in which phase last
             bool ok = true;
-            for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
+            int skip = wait->skip_kb;   // test hook: that K step of the first tile is not loaded
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step, skip = -1) {
                 int tm, tn;
                 coords(t, tm, tn);
                 const uint64_t msk = tile_mask(tm, tn);
                 const int nkb = tile_num_kb(msk);
                 uint64_t rest = msk;
                 int kidx = 0;
+                // the CTA's rows of the tile's operands
+                const int xa = kAMN ? mn_coord((int64_t)tm * BM, g.m, g.mn_remap & 1) : tm * BM;
+                const int xb = kBMN ? mn_coord((int64_t)tn * BN + rank * (BN / 2), g.l, g.mn_remap & 2)
+                                    : tn * BN + rank * (BN / 2);
                 for (int kb = 0, kin = 0; kb < nkb; ++kb) {
-                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, abort)) { ok = false; break; }
+                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, wait)) { ok = false; break; }
                     if (kin == 0) {
                         // the next kept sketch block of this tile
                         if (g.block_masks) {
@@ -810,30 +815,27 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
                     }
                     const int kz = kidx * g.b + kin * BKE;
                     if (++kin == g.kb_per_blk) kin = 0;
+                    if (kb == skip) {
+                        if (++stage == STAGES) stage = 0, phase ^= 1u;
+                        continue;
+                    }
                     uint8_t *st = tiles + stage * C::STAGE_BYTES;
                     const uint32_t fb = cluster_addr(&full[stage], 0);
                     if (leader) mbar_expect_tx(&full[stage], C::PAIR_TX);
-                    if constexpr (kAMN) {
-                        const int x = mn_coord((int64_t)tm * BM, g.m, g.mn_remap & 1);
-                        tma_load_4d_pair(&tmap_a, fb, st, 0, 0, x / 64, kz / 8);
-                    } else {
-                        tma_load_2d_pair(&tmap_a, fb, st, kz, tm * BM);
-                    }
-                    if constexpr (kBMN) {
-                        const int x = mn_coord((int64_t)tn * BN + rank * (BN / 2), g.l, g.mn_remap & 2);
-                        tma_load_4d_pair(&tmap_b, fb, st + C::A_BYTES, 0, 0, x / 64, kz / 8);
-                    } else {
-                        tma_load_2d_pair(&tmap_b, fb, st + C::A_BYTES, kz, tn * BN + rank * (BN / 2));
-                    }
-                    issued[stage] = true;
-                    issued_phase[stage] = phase;
+                    if constexpr (kAMN) tma_load_4d_pair(&tmap_a, fb, st, 0, 0, xa / 64, kz / 8);
+                    else tma_load_2d_pair(&tmap_a, fb, st, kz, xa);
+                    if constexpr (kBMN) tma_load_4d_pair(&tmap_b, fb, st + C::A_BYTES, 0, 0, xb / 64, kz / 8);
+                    else tma_load_2d_pair(&tmap_b, fb, st + C::A_BYTES, kz, xb);
+                    issued |= 1u << stage;
+                    issued_phase = (issued_phase & ~(1u << stage)) | phase << stage;
                     if (++stage == STAGES) stage = 0, phase ^= 1u;
                 }
             }
             // every stage this CTA loaded has been consumed by the pair's MMAs (so its
             // copies have landed and no commit is still on its way here)
             for (int s = 0; ok && s < STAGES; ++s)
-                if (issued[s] && !mbar_wait_cluster(&empty[s], issued_phase[s], abort)) ok = false;
+                if ((issued >> s & 1u) && !mbar_wait_cluster(&empty[s], issued_phase >> s & 1u, wait)) ok = false;
+            if (!ok) drain_pair_copies<STAGES>(leader, full, empty, drain, issued, issued_phase, wait);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader; one lane issues, the warp waits together) ----------------
@@ -849,14 +851,14 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
                 int tm, tn;
                 coords(t, tm, tn);
                 const int nkb = tile_num_kb(tile_mask(tm, tn));
-                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, abort))) {
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, wait))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t d = tmem_base + (uint32_t)(a * BN);
                 for (int kb = 0; kb < nkb; ++kb) {
-                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort))) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, wait))) { ok = false; break; }
                     tc_fence_after();
                     if (elect_one()) {
                         const uint32_t sa0 = smem_u32(tiles + stage * C::STAGE_BYTES);
@@ -882,7 +884,7 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
             }
             if (!ok && any && elect_one()) {
                 // drain: wait for the MMAs already issued before TMEM is freed
-                umma_commit_pair(drain, 0x1);
+                umma_commit_pair(drain, 0x3);
                 mbar_wait_drain(drain, 0);
             }
         }
@@ -899,7 +901,7 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
             coords(t, tm, tn);
             const int a = iter & 1;
             const uint32_t aphase = (uint32_t)(iter >> 1) & 1u;
-            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, abort))) break;
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, wait))) break;
             tc_fence_after();
             const int64_t r = (int64_t)tm * BM + row_in_tile;
             const int64_t c0 = (int64_t)tn * BN;
@@ -994,8 +996,8 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
     uint64_t *tmem_empty = tmem_full + 2;                                          // leader's are used
     uint64_t *cross_empty = tmem_empty + 2;                                        // leader's is used
     uint64_t *drain = cross_empty + 1;
-    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 1);
-    volatile int *abort = reinterpret_cast<volatile int *>(tmem_base_slot + 1);
+    volatile WaitState *wait = reinterpret_cast<volatile WaitState *>(drain + 1);
+    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 3);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)cluster_ctarank();
@@ -1014,17 +1016,18 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
         }
         mbar_init(cross_empty, 2 * 128);
         mbar_init(drain, 1);
-        *abort = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap_ah);
         prefetch_tmap(&tmap_al);
         prefetch_tmap(&tmap_bh);
         prefetch_tmap(&tmap_bl);
     }
+    if (threadIdx.x == 64) wait_state_init(wait);
     if (warp == 1) tmem_alloc_pair(tmem_base_slot, C::TMEM_COLS);
     tc_fence_before();
     cluster_sync_all();   // both CTAs' barriers exist before any remote arrival
     tc_fence_after();
+    if (threadIdx.x == 64) wait_state_taken(wait);
     const uint32_t tmem_base = *tmem_base_slot;
 
     auto coords = [&](int t, int &tm, int &tn) {
@@ -1038,16 +1041,19 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
         if (lane == 0) {
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t issued_phase[STAGES];
-            bool issued[STAGES];
-            for (int s = 0; s < STAGES; ++s) issued[s] = false, issued_phase[s] = 0;
+            uint32_t issued = 0, issued_phase = 0;   // bit s: stage s was loaded, and in which phase last
             bool ok = true;
-            for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
+            int skip = wait->skip_kb;   // test hook: that K step of the first tile is not loaded
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step, skip = -1) {
                 int tm, tn;
                 coords(t, tm, tn);
                 const int brow = tn * BN + rank * (BN / 2);
                 for (int kb = 0; kb < g.num_kb; ++kb) {
-                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, abort)) { ok = false; break; }
+                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, wait)) { ok = false; break; }
+                    if (kb == skip) {
+                        if (++stage == STAGES) stage = 0, phase ^= 1u;
+                        continue;
+                    }
                     const int blk = kb / g.kb_per_blk;
                     const int kz = g.kept.idx[blk] * g.b + (kb - blk * g.kb_per_blk) * C::BKE;
                     uint8_t *st = tiles + stage * C::STAGE_BYTES;
@@ -1057,15 +1063,16 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                     tma_load_2d_pair(&tmap_al, fb, st + C::A_BYTES, kz, tm * BM);
                     tma_load_2d_pair(&tmap_bh, fb, st + 2 * C::A_BYTES, kz, brow);
                     tma_load_2d_pair(&tmap_bl, fb, st + 2 * C::A_BYTES + C::B_BYTES, kz, brow);
-                    issued[stage] = true;
-                    issued_phase[stage] = phase;
+                    issued |= 1u << stage;
+                    issued_phase = (issued_phase & ~(1u << stage)) | phase << stage;
                     if (++stage == STAGES) stage = 0, phase ^= 1u;
                 }
             }
             // every stage this CTA loaded has been consumed by the pair's MMAs (so its
             // copies have landed and no commit is still on its way here)
             for (int s = 0; ok && s < STAGES; ++s)
-                if (issued[s] && !mbar_wait_cluster(&empty[s], issued_phase[s], abort)) ok = false;
+                if ((issued >> s & 1u) && !mbar_wait_cluster(&empty[s], issued_phase >> s & 1u, wait)) ok = false;
+            if (!ok) drain_pair_copies<STAGES>(leader, full, empty, drain, issued, issued_phase, wait);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader; one lane issues, the warp waits together) ----------------
@@ -1077,7 +1084,7 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
             bool any = false;
             const uint32_t dx = tmem_base + (uint32_t)C::CROSS;
             for (int t = t_first; ok && t < g.num_tiles; t += t_step, ++tile) {
-                if (!__all_sync(0xffffffffu, mbar_wait_cluster(cross_empty, (uint32_t)(tile & 1) ^ 1u, abort))) {
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(cross_empty, (uint32_t)(tile & 1) ^ 1u, wait))) {
                     ok = false;
                     break;
                 }
@@ -1085,14 +1092,14 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                     const int kc_end = min(g.num_kb, kc + C::CHUNK_KB);
                     const int a = chunk & 1;
                     const uint32_t aphase = (uint32_t)(chunk >> 1) & 1u;
-                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, abort))) {
+                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, wait))) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
                     const uint32_t d = tmem_base + (uint32_t)(a * BN);
                     for (int kb = kc; kb < kc_end; ++kb) {
-                        if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort))) { ok = false; break; }
+                        if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, wait))) { ok = false; break; }
                         tc_fence_after();
                         if (elect_one()) {
                             const uint32_t sah = smem_u32(tiles + stage * C::STAGE_BYTES);
@@ -1122,7 +1129,7 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
             }
             if (!ok && any && elect_one()) {
                 // drain: wait for the MMAs already issued before TMEM is freed
-                umma_commit_pair(drain, 0x1);
+                umma_commit_pair(drain, 0x3);
                 mbar_wait_drain(drain, 0);
             }
         }
@@ -1146,7 +1153,7 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                 const int a = chunk & 1;
                 const uint32_t aphase = (uint32_t)(chunk >> 1) & 1u;
                 // warp-uniform decision: tcgen05.ld below is a .sync.aligned instruction
-                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, abort))) { ok = false; break; }
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, wait))) { ok = false; break; }
                 tc_fence_after();
                 if (kc + C::CHUNK_KB >= g.num_kb) {
                     // the tile's last chunk: the cross terms are complete too
@@ -1249,8 +1256,8 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     uint64_t *tmem_full = sf_empty + SLOTS;
     uint64_t *tmem_empty = tmem_full + 2;                                          // leader's are used
     uint64_t *drain = tmem_empty + 2;
-    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 1);
-    volatile int *abort = reinterpret_cast<volatile int *>(tmem_base_slot + 1);
+    volatile WaitState *wait = reinterpret_cast<volatile WaitState *>(drain + 1);
+    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(drain + 3);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = (int)cluster_ctarank();
@@ -1273,15 +1280,16 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             mbar_init(&tmem_empty[a], 2 * 128);   // the epilogue threads of both CTAs
         }
         mbar_init(drain, 1);
-        *abort = 0;
         fence_barrier_init();
         prefetch_tmap(&tmap_a);
         prefetch_tmap(&tmap_b);
     }
+    if (threadIdx.x == 64) wait_state_init(wait);
     if (warp == 1) tmem_alloc_pair(tmem_base_slot, C::TMEM_COLS);
     tc_fence_before();
     cluster_sync_all();   // both CTAs' barriers exist before any remote arrival
     tc_fence_after();
+    if (threadIdx.x == 64) wait_state_taken(wait);
     const uint32_t tmem_base = *tmem_base_slot;
 
     auto coords = [&](int t, int &tm, int &tn) {
@@ -1295,15 +1303,18 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
         if (elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
-            uint32_t issued_phase[STAGES];
-            bool issued[STAGES];
-            for (int s = 0; s < STAGES; ++s) issued[s] = false, issued_phase[s] = 0;
+            uint32_t issued = 0, issued_phase = 0;   // bit s: stage s was loaded, and in which phase last
             bool ok = true;
-            for (int t = t_first; ok && t < g.num_tiles; t += t_step) {
+            int skip = wait->skip_kb;   // test hook: that K step of the first tile is not loaded
+            for (int t = t_first; ok && t < g.num_tiles; t += t_step, skip = -1) {
                 int tm, tn;
                 coords(t, tm, tn);
                 for (int kb = 0; kb < g.num_kb; kb += C::STAGE_KB) {
-                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, abort)) { ok = false; break; }
+                    if (!mbar_wait_cluster(&empty[stage], phase ^ 1u, wait)) { ok = false; break; }
+                    if (skip >= kb && skip < kb + C::STAGE_KB) {
+                        if (++stage == STAGES) stage = 0, phase ^= 1u;
+                        continue;
+                    }
                     const int steps = min(C::STAGE_KB, g.num_kb - kb);
                     uint8_t *st = tiles + stage * C::STAGE_BYTES;
                     const uint32_t fb = cluster_addr(&full[stage], 0);
@@ -1317,15 +1328,16 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
                         tma_load_2d_pair(&tmap_a, fb, st + q * C::STEP_BYTES, kz, tm * BM);
                         tma_load_2d_pair(&tmap_b, fb, st + q * C::STEP_BYTES + C::A_BYTES, kz, tn * BN + rank * (BN / 2));
                     }
-                    issued[stage] = true;
-                    issued_phase[stage] = phase;
+                    issued |= 1u << stage;
+                    issued_phase = (issued_phase & ~(1u << stage)) | phase << stage;
                     if (++stage == STAGES) stage = 0, phase ^= 1u;
                 }
             }
             // every stage this CTA loaded has been consumed by the pair's MMAs (so its
             // copies have landed and no commit is still on its way here)
             for (int s = 0; ok && s < STAGES; ++s)
-                if (issued[s] && !mbar_wait_cluster(&empty[s], issued_phase[s], abort)) ok = false;
+                if ((issued >> s & 1u) && !mbar_wait_cluster(&empty[s], issued_phase >> s & 1u, wait)) ok = false;
+            if (!ok) drain_pair_copies<STAGES>(leader, full, empty, drain, issued, issued_phase, wait);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader; one lane issues, the warp waits together) ----------------
@@ -1338,7 +1350,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             for (int t = t_first; ok && t < g.num_tiles; t += t_step, ++iter) {
                 const int a = iter & 1;
                 const uint32_t aphase = (uint32_t)(iter >> 1) & 1u;
-                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, abort))) {
+                if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_empty[a], aphase ^ 1u, wait))) {
                     ok = false;
                     break;
                 }
@@ -1347,7 +1359,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
                 for (int kb = 0; kb < g.num_kb; kb += C::STAGE_KB) {
                     const uint32_t sfa = tmem_base + C::sfa(slot), sfb = sfa + 4;
                     if (kb % C::GROUP_KB == 0) {
-                        if (!__all_sync(0xffffffffu, mbar_wait_cluster(&sf_ready[slot], sphase, abort))) { ok = false; break; }
+                        if (!__all_sync(0xffffffffu, mbar_wait_cluster(&sf_ready[slot], sphase, wait))) { ok = false; break; }
                         tc_fence_after();
                         if (elect_one()) {
                             const uint32_t ch = smem_u32(chunks + slot * C::CHUNKS * 512);
@@ -1358,7 +1370,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
                         __syncwarp();
                         any = true;
                     }
-                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, abort))) { ok = false; break; }
+                    if (!__all_sync(0xffffffffu, mbar_wait_cluster(&full[stage], phase, wait))) { ok = false; break; }
                     tc_fence_after();
                     const int next = kb + C::STAGE_KB;
                     const bool last = next % C::GROUP_KB == 0 || next >= g.num_kb;   // of the scale group
@@ -1388,7 +1400,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             }
             if (!ok && any && elect_one()) {
                 // drain: wait for the MMAs already issued before TMEM is freed
-                umma_commit_pair(drain, 0x1);
+                umma_commit_pair(drain, 0x3);
                 mbar_wait_drain(drain, 0);
             }
         }
@@ -1424,7 +1436,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
                     w[u] |= (ue8m0_x4(f) & 0xffu) << (8 * q);
                 }
             }
-            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&sf_empty[slot], phase ^ 1u, abort))) { ok = false; break; }
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&sf_empty[slot], phase ^ 1u, wait))) { ok = false; break; }
 #pragma unroll
             for (int c = 0; c < C::CHUNKS; ++c)
                 *reinterpret_cast<uint4 *>(ch + 512 * c + 16 * lane) =
@@ -1434,7 +1446,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             if (lane == 0) mbar_arrive_cluster(ready);
         }
         // the last group of this slot has been consumed: no commit is still on its way here
-        if (ok && it > slot) mbar_wait_cluster(&sf_empty[slot], phase ^ 1u, abort);
+        if (ok && it > slot) mbar_wait_cluster(&sf_empty[slot], phase ^ 1u, wait);
     } else {
         // ---------------- epilogue (warps 2..5): this CTA's 128 rows ----------------
         const int quarter = warp & 3;
@@ -1448,7 +1460,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             coords(t, tm, tn);
             const int a = iter & 1;
             const uint32_t aphase = (uint32_t)(iter >> 1) & 1u;
-            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, abort))) break;
+            if (!__all_sync(0xffffffffu, mbar_wait_cluster(&tmem_full[a], aphase, wait))) break;
             tc_fence_after();
             const int64_t r0 = (int64_t)tm * BM + quarter * 32, c0 = (int64_t)tn * BN;
             for (int ch = 0; ch < BN / 32; ++ch) {

@@ -18,9 +18,9 @@ __device__ unsigned int g_device_status;
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;   // 1 s per wait
 
 // Test hook of the bounded waits (oversketch_test_wait_timeout): when >= 0, the
-// next launch of gemm_masked_tc_kernel takes this value (one-shot) and its first
-// CTA leaves that K step of its first tile unloaded, with g_test_wait_ns as the
-// CTA's wait limit, so that the wait for that stage runs out.
+// next launch of a GEMM kernel of gemm_tc.cu takes this value (one-shot) and its
+// first CTA (or CTA pair) leaves that K step of its first tile unloaded, with
+// g_test_wait_ns as its wait limit, so that the wait for that stage runs out.
 __device__ int g_test_skip_kb = -1;
 __device__ unsigned long long g_test_wait_ns = kWaitLimitNs;
 
@@ -83,10 +83,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
 }
 
 // Same, but ignores the abort flag (used while draining in-flight copies).
-__device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity,
+                                                unsigned long long limit_ns = kWaitLimitNs) {
     const unsigned long long t0 = globaltimer_ns();
     while (!mbar_try_wait(bar, parity)) {
-        if (globaltimer_ns() - t0 > kWaitLimitNs) {
+        if (globaltimer_ns() - t0 > limit_ns) {
             atomicOr(&g_device_status, 1u);
             return false;
         }
@@ -193,16 +194,40 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t *bar, uint32_t pa
     return ok != 0;
 }
 
+// What the roles of a pair's CTA share about its waits, in shared memory: the abort
+// flag, and from the test hook the K step to leave out (-1: none) and the limit.
+struct WaitState {
+    int abort, skip_kb;
+    unsigned long long limit_ns;
+};
+
+// Set by one thread of each CTA before the pair's first cluster barrier: both CTAs of
+// the first pair see the same hook.  wait_state_taken, after that barrier, consumes it.
+__device__ __forceinline__ void wait_state_init(volatile WaitState *w) {
+    int skip = -1;
+    unsigned long long limit = kWaitLimitNs;
+    if (blockIdx.x < 2) {
+        skip = *(volatile int *)&g_test_skip_kb;
+        if (skip >= 0) limit = *(volatile unsigned long long *)&g_test_wait_ns;
+    }
+    w->abort = 0;
+    w->skip_kb = skip;
+    w->limit_ns = limit;
+}
+__device__ __forceinline__ void wait_state_taken(volatile WaitState *w) {
+    if (blockIdx.x == 0 && w->skip_kb >= 0) g_test_skip_kb = -1;
+}
+
 // Bounded wait as mbar_wait, at cluster scope.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, volatile int *abort) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t *bar, uint32_t parity, volatile WaitState *w) {
     if (mbar_try_wait_cluster(bar, parity)) return true;
     const unsigned long long t0 = globaltimer_ns();
     for (uint32_t it = 1;; ++it) {
         if (mbar_try_wait_cluster(bar, parity)) return true;
         if ((it & 63u) == 0) {
-            if (*abort) return false;
-            if (globaltimer_ns() - t0 > kWaitLimitNs) {
-                *abort = 1;
+            if (w->abort) return false;
+            if (globaltimer_ns() - t0 > w->limit_ns) {
+                w->abort = 1;
                 atomicOr(&g_device_status, 1u);
                 return false;
             }
@@ -226,6 +251,25 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t *bar, uint16_t cta_mas
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
                  ::"r"(smem_u32(bar)), "h"(cta_mask)
                  : "memory");
+}
+
+// (Bit s of issued / phase: stage s was loaded, and in which phase last.)
+// A pair's producer that gave up waits for its copies in flight before the CTA may free
+// its tensor memory and end.  The leader's barriers count both CTAs' copies: it waits for
+// the stages it armed.  The other CTA has no barrier for its copies alone: it waits until
+// the leader's last MMAs are done and its stages consumed, or for the wait limit, which no
+// copy takes.
+template <int STAGES>
+__device__ __forceinline__ void drain_pair_copies(bool leader, uint64_t *full, uint64_t *empty, uint64_t *drain,
+                                                  uint32_t issued, uint32_t phase, volatile WaitState *w) {
+    if (leader) {
+        for (int s = 0; s < STAGES; ++s)
+            if (issued >> s & 1u) mbar_wait_drain(&full[s], phase >> s & 1u);
+        return;
+    }
+    bool in_time = mbar_wait_drain(drain, 0, w->limit_ns);
+    for (int s = 0; s < STAGES; ++s)
+        if (in_time && (issued >> s & 1u)) in_time = mbar_wait_drain(&empty[s], phase >> s & 1u, w->limit_ns);
 }
 
 // TMEM allocation shared by the pair: one warp of each CTA executes it.

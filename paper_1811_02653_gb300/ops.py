@@ -545,8 +545,8 @@ def device_status(reset=True, stream=None) -> int:
 
 
 def test_wait_timeout(limit_ns: int, skip_kb: int):
-    """Test hook: the next one-CTA tensor-core GEMM launch leaves K step skip_kb of
-    its first tile unloaded and gives up after limit_ns (skip_kb < 0 withdraws it)."""
+    """Test hook: the next tensor-core GEMM launch leaves K step skip_kb of its first
+    tile unloaded and gives up after limit_ns (skip_kb < 0 withdraws it)."""
     _check(load_library().oversketch_test_wait_timeout(limit_ns, skip_kb), "oversketch_test_wait_timeout")
 
 

@@ -534,6 +534,7 @@ namespace {
 // padded to a multiple of 64), and the K-major copies are not made.
 struct BackwardLayout {
     bool mn;                         // operands read MN-major (no transposed copies)
+    bool tall;                       // T^T's pitch is past the row gather's: T instead, kb columns
     int64_t kb, ld_l, ld_m, ld_t;    // padded row pitches (elements) of the BF16 / FP32 buffers
     size_t dc16, bsel, t, asel, dct16, u;
 };
@@ -545,9 +546,10 @@ BackwardLayout backward_layout(const Plan *p, int64_t m, int64_t l, uint64_t mas
     L.ld_l = L.mn ? (l + 63) / 64 * 64 : (l + 7) / 8 * 8;   // BF16 rows of l elements
     L.ld_m = (m + 7) / 8 * 8;      // BF16 rows of m elements
     L.ld_t = (m + 3) / 4 * 4;      // FP32 rows of m elements (T transposed)
+    L.tall = !L.mn && L.ld_t >= (int64_t(1) << 30);
     L.dc16 = align256((size_t)m * L.ld_l * 2);
     L.bsel = L.mn ? 0 : align256((size_t)L.kb * L.ld_l * 2);
-    L.t = align256((size_t)L.kb * L.ld_t * 4);
+    L.t = L.tall ? align256((size_t)m * ((L.kb + 3) / 4 * 4) * 4) : align256((size_t)L.kb * L.ld_t * 4);
     L.asel = L.mn ? 0 : align256((size_t)L.kb * L.ld_m * 2);
     L.dct16 = L.mn ? 0 : align256((size_t)l * L.ld_m * 2);
     L.u = align256((size_t)L.kb * ((l + 3) / 4 * 4) * 4);
@@ -600,7 +602,16 @@ extern "C" os_status oversketch_matmul_backward(oversketch_plan_t plan, const vo
         float *Tt = reinterpret_cast<float *>(base + L.bsel);
         base += L.bsel + L.t;
         // T^T = B~_sel dC^T (kb x m): its rows are what the gather into dX reads
-        if (l > 0 && L.mn) {
+        if (L.tall) {
+            const int64_t ld = (L.kb + 3) / 4 * 4;
+            if (l > 0) {
+                OSK_TRY(oversketch_select_transpose(BtT, OS_BF16, l, z, ldbt, mask, p->b, bsel, OS_BF16, L.ld_l, stream));
+                OSK_TRY(oversketch_gemm_bf16(dc16, L.ld_l, bsel, L.ld_l, m, L.kb, l, inv_k, 0.0f, Tt, ld, stream));
+            } else {
+                OSK_CUDA_TRY(cudaMemsetAsync(Tt, 0, (size_t)m * ld * 4, st));
+            }
+            OSK_TRY(oversketch_unsketch_cols(plan, Tt, m, ld, mask, 1.0f, dX, x_t, ldx, stream));
+        } else if (l > 0 && L.mn) {
             // B~^T (l x z) read MN-major, kept blocks picked by column
             OSK_TRY(gemm_bf16_mn(BtT, ldbt, true, dc16, L.ld_l, false, L.kb, m, l, inv_k, Tt, L.ld_t, p->b, 1, mask,
                                  p->P, st));
@@ -610,7 +621,7 @@ extern "C" os_status oversketch_matmul_backward(oversketch_plan_t plan, const vo
         } else {
             OSK_CUDA_TRY(cudaMemsetAsync(Tt, 0, (size_t)L.kb * L.ld_t * 4, st));
         }
-        OSK_TRY(unsketch_cols_t_impl(p, Tt, m, L.ld_t, mask, dX, x_t, ldx, st));
+        if (!L.tall) OSK_TRY(unsketch_cols_t_impl(p, Tt, m, L.ld_t, mask, dX, x_t, ldx, st));
     }
     if (need_dg) {
         if (m > 0 && !At) return OS_ERR_INVALID_ARG;

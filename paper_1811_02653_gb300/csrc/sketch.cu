@@ -840,7 +840,7 @@ __global__ void __launch_bounds__(256, 4) unsketch_cols_t_kernel(
     __shared__ float4 tile[kUtRows][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t i0 = (int64_t)blockIdx.x * kUtRows, r0 = (int64_t)blockIdx.y * 128;
-    const bool live = r0 + 4 * lane < ldt;               // the pitch is a multiple of 4 that holds m
+    const bool live = r0 + 4 * lane < m;                 // the pitch is a multiple of 4 that holds m
     const uint64_t base = reinterpret_cast<uint64_t>(Tt + (live ? r0 + 4 * lane : r0));
     const uint32_t row_bytes = (uint32_t)(4 * ldt);      // the launch keeps 4 ldt below 2^32
     const uint64_t block_bytes = (uint64_t)b * row_bytes;
@@ -1451,18 +1451,23 @@ os_status unsketch_rows_impl(const Plan *p, const float *U, int64_t l, int64_t l
     return check_launch();
 }
 
-// dX (m x n) from the transposed kept blocks Tt (kb x m, pitch ldt a multiple of 4).
+// dX (m x n) from the transposed kept blocks Tt (kb x m, pitch ldt < 2^30, a multiple of 4).
 os_status unsketch_cols_t_impl(const Plan *p, const float *Tt, int64_t m, int64_t ldt, uint64_t mask, void *dX,
                                os_dtype x_t, int64_t ldx, cudaStream_t st) {
     const BlockList kept = mask_to_list(mask, p->P);
-    const dim3 grid((unsigned)((p->n + kUtRows - 1) / kUtRows), (unsigned)((m + 127) / 128));
-    if (grid.y > 65535u || ldt % 4 != 0 || ldt >= (int64_t(1) << 30) || !aligned16(Tt)) return OS_ERR_UNSUPPORTED;
+    if (ldt % 4 != 0 || ldt >= (int64_t(1) << 30) || !aligned16(Tt)) return OS_ERR_UNSUPPORTED;
     auto launch = [&](auto *out) -> os_status {
         using O = typename std::remove_pointer<decltype(out)>::type;
         const bool vec = aligned16(dX) && (ldx * (int64_t)sizeof(O)) % 16 == 0;
         auto k = vec ? unsketch_cols_t_kernel<O, true> : unsketch_cols_t_kernel<O, false>;
-        k<<<grid, 256, 0, st>>>(Tt, m, ldt, p->hs, p->n, p->b, kept, out, ldx);
-        return check_launch();
+        constexpr int64_t kRows = 65535 * int64_t(128);   // rows of dX per launch (grid.y)
+        for (int64_t r = 0; r < m; r += kRows) {
+            const int64_t rows = m - r < kRows ? m - r : kRows;
+            const dim3 grid((unsigned)((p->n + kUtRows - 1) / kUtRows), (unsigned)((rows + 127) / 128));
+            k<<<grid, 256, 0, st>>>(Tt + r, rows, ldt, p->hs, p->n, p->b, kept, out + r * ldx, ldx);
+            OSK_TRY(check_launch());
+        }
+        return OS_OK;
     };
     return x_t == OS_F32 ? launch((float *)dX) : launch((__nv_bfloat16 *)dX);
 }

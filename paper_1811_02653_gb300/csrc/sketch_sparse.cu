@@ -23,7 +23,8 @@
 //      FP8 with the per-128-column UE8M0 scale, FP32, or TF32 hi/lo planes).  No
 //      float atomics: bitwise reproducible.
 //   Two groups of 512 threads share a CTA and take turns at the routing, so that one
-//   row streams from HBM while the other is routed; the bucket tables exist once.
+//   row streams from HBM while the other is routed; the bucket tables exist once.  Rows
+//   of many nonzeros are taken one at a time by all 1024 threads (sp1_groups).
 //   A row with more nonzeros in some warp's share than a region holds is left to the
 //   flushing kernel: its first kept output gets a marker value.
 //   Bound by HBM and instruction issue together.  4096 x 2^20 FP32 at 1 % (17.2 GB,
@@ -427,6 +428,9 @@ template <int NG> struct Sp1 {
     static constexpr int kMaxPairs = 16;                // codes of a lane's entries, two per register
     static constexpr int kMaxRegion = 64 * kMaxPairs;   // entries per warp
     static constexpr size_t kFixed = sizeof(uint32_t) * (kSp1MaxBuckets / 2 + 40 * NG) + 16;
+    static constexpr int kFits = (int)((kSmemLimit - kFixed - 64) / (GW * kEntryBytes) / 4 * 4);
+    static constexpr int kRegion = kFits < kMaxRegion ? kFits : kMaxRegion;   // entries per warp that there is room for
+    static constexpr size_t kSmem = kFixed + (size_t)kEntryBytes * GW * kRegion;
     static_assert(kMaxRegion * GW <= 32768, "entry numbers have 15 bits");
 };
 
@@ -881,20 +885,19 @@ __device__ __forceinline__ typename RowMark<OutT>::U *row_mark(OutT *At, int64_t
     return reinterpret_cast<typename RowMark<OutT>::U *>(At + r * ldat + col);
 }
 
-// The one-pass kernel (persistent over rows).  Group g of a CTA takes every NG-th of
-// its rows; with two groups the routing (the shared counters and entry lists) goes
-// from one to the other row by row, so each group compacts while the other routes.
-// A row whose nonzeros overflow a warp's region is marked for the flushing kernel.
+// The CTA's rows.  Group g takes every NG-th of them; with two groups the routing (the
+// shared counters and entry lists) goes from one to the other row by row, so each group
+// compacts while the other routes.  A row whose nonzeros overflow a warp's region is
+// marked for the flushing kernel.
 template <typename InT, typename OutT, bool kScale, int NG>
-__global__ void __launch_bounds__(kSpThreads, 1)
-sketch_left_onepass_kernel(const InT *__restrict__ A, int64_t lda, int64_t m, int64_t n, bool vec,
-                           const uint32_t *__restrict__ hs, uint64_t seed, bool hashed, int32_t b,
-                           const __grid_constant__ BlockList blocks, int cw,
-                           const float *__restrict__ col_scale, OutT *__restrict__ At, int64_t ldat,
-                           float *__restrict__ scales, int64_t lds, int64_t plane_elems) {
+__device__ __forceinline__ void sp1_rows(const InT *__restrict__ A, int64_t lda, int64_t rows, int64_t n, bool vec,
+                                         const uint32_t *__restrict__ hs, uint64_t seed, bool hashed, int32_t b,
+                                         const BlockList &blocks, const float *__restrict__ col_scale,
+                                         OutT *__restrict__ At, int64_t ldat, float *__restrict__ scales, int64_t lds,
+                                         int64_t plane_elems, float4 *sp_smem) {
     using S = Sp1<NG>;
     using Idx = typename S::Idx;
-    extern __shared__ float4 sp_smem[];
+    constexpr int cw = S::kRegion;
     const int ge = S::GW * cw;                      // entries per group
     uint32_t cnt;                                   // kSp1MaxBuckets / 2 words, then 40 words per group for the scan
     asm volatile("mov.u32 %0, %1;" : "=r"(cnt) : "r"((uint32_t)__cvta_generic_to_shared(sp_smem)));
@@ -908,7 +911,6 @@ sketch_left_onepass_kernel(const InT *__restrict__ A, int64_t lda, int64_t m, in
     const uint32_t wval = val + 4 * warp * cw, widx = idx + (uint32_t)sizeof(Idx) * warp * cw;   // the warp's region
     const int64_t seg = ((n + S::GW - 1) / S::GW + 1023) / 1024 * 1024;   // columns per warp: whole steps
     const int64_t s0 = min(n, (int64_t)warp * seg), s1 = min(n, s0 + seg);
-    const int64_t rows = (m - blockIdx.x + gridDim.x - 1) / gridDim.x;   // of this CTA
     for (int64_t q = g; q < rows; q += NG) {
         const int64_t r = blockIdx.x + q * gridDim.x;
         const int have = sp1_compact<InT, Idx>(A + r * lda, s0, s1, vec, wval, widx, cw);
@@ -932,6 +934,109 @@ sketch_left_onepass_kernel(const InT *__restrict__ A, int64_t lda, int64_t m, in
     }
 }
 
+// Nonzeros (x) among the elements (y) of 4 pieces of 16 bytes per thread, over the CTA:
+// piece q of a thread is at place(q).x in row place(q).y of A.
+template <typename InT, typename Place>
+__device__ __forceinline__ int2 sp1_sample(const InT *__restrict__ A, int64_t lda, int64_t n, bool vec, Place place,
+                                           float4 *sp_smem) {
+    using P = Piece<InT>;
+    constexpr int Q = 4, E = P::E;
+    uint32_t *sums = reinterpret_cast<uint32_t *>(sp_smem);
+    uint4 u[Q];
+    uint32_t s = 0;   // both counts stay below 2^16 over the CTA
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        const longlong2 at = place(q);
+        u[q] = make_uint4(0u, 0u, 0u, 0u);
+        if (at.x + E > n) continue;
+        s += E << 16;
+        const InT *from = A + at.y * lda + at.x;
+        if (vec) {
+            u[q] = __ldg(reinterpret_cast<const uint4 *>(from));
+        } else {
+            InT e[E];
+#pragma unroll
+            for (int j = 0; j < E; ++j) e[j] = from[j];
+            u[q] = *reinterpret_cast<const uint4 *>(e);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) s += __popc(P::mask(u[q]));
+    s = __reduce_add_sync(0xffffffffu, s);
+    if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = __reduce_add_sync(0xffffffffu, sums[threadIdx.x & 31]);
+    __syncthreads();   // the shared memory is free
+    return make_int2((int)(s & 0xffffu), (int)(s >> 16));
+}
+
+// How the CTA takes its rows: two at a time, one, or none (0: all left to the flushing
+// kernel), by the nonzeros a row has, estimated from 64 pieces of 512 bytes of each of its
+// first two rows.  Two groups hide the streaming of one row behind the routing of
+// another, but route with half the threads and hold fewer entries: 996 in each 16th of a
+// row against 700 in each 32nd, so that uniform rows of 2^20 columns overflow from 1.44 %
+// and from 1.85 % on, and a row that does is read twice.  us on GB300, two groups / one:
+// 2048 rows of 2^20, b = 2048: 1 % 2655 / 2468, 1.35 % 3796 / 3091, 1.44 % 7534 / 3244,
+// 1.6 % 6563 / 3523; 1216 rows, b = 4096: 0.6 % 920 / 1093, 1.2 % 1403 / 1484; 608 rows of
+// 2^19, b = 2048: 1.2 % 455 / 459, 2 % 753 / 656; 456 rows of 65536, b = 2048: 2 % 106 /
+// 106, 20 % 634 / 473; b = 512: 2 % 111 / 119.  Blocks below 1024 (long bucket lists) go
+// straight to the flushing kernel then: 1216 rows of 2^20 at 1.44 %, b = 256: one group
+// 7.3 ms, flushed 5.0.  Where rows may overflow every CTA takes the same larger sample of all
+// of A: some leaving their rows and some not would wait for each other in both kernels.
+// Not inlined: the row loops' registers are allocated 2 % better without it.
+template <typename InT>
+__device__ __noinline__ int sp1_groups(const InT *__restrict__ A, int64_t lda, int64_t m, int64_t rows, int64_t n,
+                                          int32_t b, bool vec, float4 *sp_smem) {
+    constexpr int E = Piece<InT>::E;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t seg = ((n + 15) / 16 + 1023) / 1024 * 1024, s0 = (warp & 15) * seg;
+    const int64_t r = blockIdx.x + (rows > 1 ? (int64_t)(warp >> 4) * gridDim.x : 0);
+    // the shares' first steps come into L2 meanwhile
+    if (vec && lane == 0 && s0 + 3 * 128 * E <= n) l2_prefetch(A + r * lda + s0, 3 * 128 * E * (uint32_t)sizeof(InT));
+    int2 s = sp1_sample<InT>(A, lda, n, vec,
+                             [&](int q) { return make_longlong2(s0 + q * (seg / 4) + E * lane, r); }, sp_smem);
+    auto more_than = [&](int64_t entries) { return s.x * n > entries * s.y; };   // a row
+    if (more_than(11264)) {
+        s = make_int2(0, 0);
+#pragma unroll 1
+        for (int k0 = 0; k0 < 2 * 4 * kSpThreads; k0 += 4 * kSpThreads) {
+            // rows in order, columns scattered
+            const int2 part = sp1_sample<InT>(A, lda, n, vec, [&](int q) {
+                const uint32_t k = (uint32_t)k0 + threadIdx.x * 4 + q;
+                return make_longlong2((int64_t)((uint64_t)(k * 0x9E3779B1u) * (uint64_t)n >> 32) & ~int64_t(E - 1),
+                                      (int64_t)((uint64_t)k * (uint64_t)m / (8 * kSpThreads)));
+            }, sp_smem);
+            s.x += part.x;
+            s.y += part.y;
+        }
+    }
+    if (more_than(b < 1024 ? 14336 : 19456)) return 0;
+    if (b >= 1024 && more_than(b <= 3072 ? 12288 : 13312)) return 1;
+    return rows < 2 || (b >= 1024 && more_than(n / 64)) ? 1 : 2;
+}
+
+// The one-pass kernel (persistent over rows), with kTwo in two groups where that pays.
+template <typename InT, typename OutT, bool kScale, bool kTwo>
+__global__ void __launch_bounds__(kSpThreads, 1)
+sketch_left_onepass_kernel(const InT *__restrict__ A, int64_t lda, int64_t m, int64_t n, bool vec,
+                           const uint32_t *__restrict__ hs, uint64_t seed, bool hashed, int32_t b,
+                           const __grid_constant__ BlockList blocks, const float *__restrict__ col_scale,
+                           OutT *__restrict__ At, int64_t ldat, float *__restrict__ scales, int64_t lds,
+                           int64_t plane_elems) {
+    extern __shared__ float4 sp_smem[];
+    const int64_t rows = (m - blockIdx.x + gridDim.x - 1) / gridDim.x;   // of this CTA
+    const int groups = kTwo ? sp1_groups<InT>(A, lda, m, rows, n, b, vec, sp_smem) : 1;
+    if (groups == 2)
+        sp1_rows<InT, OutT, kScale, 2>(A, lda, rows, n, vec, hs, seed, hashed, b, blocks, col_scale, At, ldat, scales,
+                                       lds, plane_elems, sp_smem);
+    else if (groups == 1)
+        sp1_rows<InT, OutT, kScale, 1>(A, lda, rows, n, vec, hs, seed, hashed, b, blocks, col_scale, At, ldat, scales,
+                                       lds, plane_elems, sp_smem);
+    else
+        for (int64_t q = threadIdx.x; q < rows; q += kSpThreads)
+            *row_mark(At, blockIdx.x + q * gridDim.x, ldat, (int64_t)blocks.idx[0] * b) = RowMark<OutT>::bits;
+}
+
 // The flushing kernel: one CTA per row (persistent over rows); with kMarked,
 // only the rows the one-pass kernel marked.
 template <typename InT, typename OutT, bool kScale, bool kMarked>
@@ -944,16 +1049,22 @@ sketch_left_sparse_kernel(const InT *__restrict__ A, int64_t lda, int64_t m, int
     extern __shared__ float4 sp_smem[];
     if constexpr (kMarked) {
         // 32 of the CTA's rows at a time: every warp reads their marks (the same
-        // ballot in every warp), then the CTA runs the marked ones
+        // ballot in every warp), then the CTA runs the marked ones.  One row of each
+        // gridDim.x consecutive ones, at a place that moves on from one set to the next, so
+        // that the rows one CTA of the one-pass kernel left are shared by many here, and so
+        // are consecutive rows.
         const int lane = threadIdx.x & 31;
-        for (int64_t base = blockIdx.x; base < m; base += (int64_t)gridDim.x * 32) {
-            const int64_t rl = base + (int64_t)lane * gridDim.x;
+        auto row_of = [&](int64_t k) -> int64_t {
+            return k * gridDim.x + (blockIdx.x + (uint64_t)k * 37u) % gridDim.x;
+        };
+        for (int64_t base = 0; base * gridDim.x < m; base += 32) {
+            const int64_t rl = row_of(base + lane);
             const bool take = rl < m && *row_mark(At, rl, ldat, (int64_t)blocks.idx[0] * b) == RowMark<OutT>::bits;
             uint32_t todo = __ballot_sync(0xffffffffu, take);
             while (todo) {
                 const int t = __ffs(todo) - 1;
                 todo &= todo - 1;
-                const int64_t r = base + (int64_t)t * gridDim.x;
+                const int64_t r = row_of(base + t);
                 sp_row_flushing<InT, OutT, kScale>(A + r * lda, r, n, vec, hs, seed, hashed, b, blocks, emax,
                                                    col_scale, At, ldat, scales, lds, plane_elems, sp_smem);
             }
@@ -999,21 +1110,15 @@ os_status launch_sparse_t(const InT *A, int64_t lda, int64_t m, int64_t n, const
     const bool onepass = p->b <= kSp1MaxBuckets;
     if (onepass) {
         const bool two = m > sp_num_sms() && n <= Sp1<2>::kMaxN;
-        auto launch = [&](auto ng) -> os_status {
-            constexpr int NG = decltype(ng)::value;
-            using S = Sp1<NG>;
-            const int64_t c = ((int64_t)kSmemLimit - (int64_t)S::kFixed - 64) / (S::GW * S::kEntryBytes) / 4 * 4;
-            const int cw = (int)(c < S::kMaxRegion ? c : S::kMaxRegion);
-            const size_t smem1 = S::kFixed + (size_t)S::kEntryBytes * S::GW * cw;
-            auto k1 = col_scale ? sketch_left_onepass_kernel<InT, OutT, true, NG>
-                                : sketch_left_onepass_kernel<InT, OutT, false, NG>;
-            OSK_CUDA_TRY(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
-            k1<<<(unsigned)grid, kSpThreads, smem1, st>>>(A, lda, m, n, vec, p->hs, p->seed, p->hashed != 0, p->b,
-                                                          blocks, cw, col_scale, (OutT *)At, ldat, scales, lds,
-                                                          plane_elems);
-            return check_launch();
-        };
-        OSK_TRY(two ? launch(std::integral_constant<int, 2>()) : launch(std::integral_constant<int, 1>()));
+        auto k1 = two ? (col_scale ? sketch_left_onepass_kernel<InT, OutT, true, true>
+                                   : sketch_left_onepass_kernel<InT, OutT, false, true>)
+                      : (col_scale ? sketch_left_onepass_kernel<InT, OutT, true, false>
+                                   : sketch_left_onepass_kernel<InT, OutT, false, false>);
+        const size_t smem1 = Sp1<1>::kSmem > Sp1<2>::kSmem ? Sp1<1>::kSmem : Sp1<2>::kSmem;
+        OSK_CUDA_TRY(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1));
+        k1<<<(unsigned)grid, kSpThreads, smem1, st>>>(A, lda, m, n, vec, p->hs, p->seed, p->hashed != 0, p->b, blocks,
+                                                      col_scale, (OutT *)At, ldat, scales, lds, plane_elems);
+        OSK_TRY(check_launch());
     }
     auto k = onepass ? (col_scale ? sketch_left_sparse_kernel<InT, OutT, true, true>
                                  : sketch_left_sparse_kernel<InT, OutT, false, true>)

@@ -39,6 +39,7 @@ os_status gemm_masked_tc(const Plan *p, const void *At, int64_t ldat, const floa
                          int64_t l, uint64_t mask, float alpha, float beta, float *C, int64_t ldc,
                          cudaStream_t st);
 double tf32x3_us(int64_t m, int64_t l, int64_t K);
+double f16x3_us(int64_t m, int64_t l, int64_t K);
 
 namespace {
 thread_local char g_last_cuda_error[256] = "no error";
@@ -117,10 +118,11 @@ MatmulLayout layout(const Plan *p, int64_t m, int64_t l, os_dtype a_t, os_dtype 
 // row, gemm_masked_f16x3) instead of on TF32 planes written by the sketches: block
 // widths that fit the 64-element K tile, scratch space for what the split leaves, and a
 // GEMM that gains more than the split and its launches cost.  On GB300 a 128 x 128
-// tile of the 3xTF32 kernel takes 19.5 ns per K (152 at once, K shared by up to eight
-// CTAs when there are few tiles: tf32x3_us), a 256 x 160 tile of the FP16 one 10.2 ns
-// per K (76 at once) and 3 us; the memory-bound split and the four extra launches
-// take 8 bytes per sum at 6 TB/s and about 16 us.  Whole products, TF32 -> FP16:
+// tile of the 3xTF32 kernel takes 19.5 ns per K (one per SM at once, K shared by up to
+// eight CTAs when there are few tiles: tf32x3_us), a 256 x 160 tile of the FP16 one 10.2
+// ns per K (one per pair of SMs at once) and 3 us (f16x3_us); the memory-bound split and
+// the four extra launches take 8 bytes per sum at 6 TB/s and about 16 us.  Whole
+// products, TF32 -> FP16:
 // 8192 x 32768 x 8192 (K = 8192) 5.39 -> 3.48 ms, 4096 x 16384 x 4096 (4096) 819 ->
 // 577 us, 3000 x 16384 x 3000 (1024) 298 -> 284, 2048 x 8192 x 2048 (2048) 172 -> 166,
 // and past the line 1024 x 16384 x 1024 (4096) 135 -> 153, 4096 x 16384 x 4096 (512)
@@ -129,10 +131,7 @@ bool f16x3_pays(const Plan *p, os_dtype gemm_dtype, int64_t m, int64_t l, uint64
     if (gemm_dtype != OS_F32 || p->b % 64 != 0) return false;
     if (scratch < (size_t)(m + l) * 4 + sizeof(SplitCtl) + 256) return false;
     const double K = (double)__builtin_popcountll(mask) * p->b;
-    auto waves = [](int64_t tiles, int at_once) { return (double)((tiles + at_once - 1) / at_once); };
-    const double tf32 = tf32x3_us(m, l, (int64_t)K);
-    const double f16 = waves((m + 255) / 256 * ((l + 159) / 160), 76) * (K * 10.2e-3 + 3.0);
-    return tf32 - f16 > 16.0 + (double)(m + l) * K * 8.0 / 6e6;
+    return tf32x3_us(m, l, (int64_t)K) - f16x3_us(m, l, (int64_t)K) > 16.0 + (double)(m + l) * K * 8.0 / 6e6;
 }
 
 // The masked product of FP32 sums stored as TF32 pairs are (sums, then a plane's

@@ -576,15 +576,16 @@ __global__ void __launch_bounds__(256) pack_cols_bf16_kernel(const __nv_bfloat16
     auto at = [](int rp, int c) { return rp * PITCH + (c & ~31) + ((c + (c >> 5)) & 31); };
     const int64_t rb = blockIdx.y, row0 = rb * 64, i0 = (int64_t)blockIdx.x * W;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    if (row0 + 64 <= m && i0 + W <= n) {
+    if (i0 + W <= n) {
         const int cv = lane & 15;
+        const uint4 none = make_uint4(0u, 0u, 0u, 0u);   // rows past m
         uint4 x[2], y[2];
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const int item = 2 * warp + u, rp = 8 * (item >> 2) + (item & 3) + 4 * (lane >> 4);
             const __nv_bfloat16 *src = A + (row0 + 2 * rp) * lda + i0 + 8 * cv;
-            x[u] = __ldg(reinterpret_cast<const uint4 *>(src));
-            y[u] = __ldg(reinterpret_cast<const uint4 *>(src + lda));
+            x[u] = row0 + 2 * rp < m ? __ldg(reinterpret_cast<const uint4 *>(src)) : none;
+            y[u] = row0 + 2 * rp + 1 < m ? __ldg(reinterpret_cast<const uint4 *>(src + lda)) : none;
         }
 #pragma unroll
         for (int u = 0; u < 2; ++u) {

@@ -980,43 +980,50 @@ os_status launch_entry_weights(const Plan *p, const float *s, uint64_t block_mas
 
 // FP8 codes and UE8M0 scales from FP32 sums staged in global memory; the same rule
 // as the gather's fused FP8 epilogue (smallest e with amax <= 448 * 2^e, codes =
-// RNE(x / 2^e)), so the codes and scales are the same bits.  A CTA takes a row at a
-// time; a warp quantises kQuant 128-column slices of it at once.  Memory-bound: one
-// slice per warp (16 bytes per lane in flight) ran at 3.2 TB/s on GB300, and the two
-// quantisations of an 8192 x 32768 x 8192 product took about 50 us longer together.
+// RNE(x / 2^e)), so the codes and scales are the same bits.  A warp quantises Q
+// consecutive 128-column slices of a row at once, the warps of the grid one after the
+// other over the slices of all rows.  Memory-bound: one slice per warp (16 bytes per lane
+// in flight) ran at 3.2 TB/s on GB300, and the two quantisations of an 8192 x 32768 x 8192
+// product took about 50 us longer together.  Q = 1 while all slices have a warp on the
+// GPU at once (left sketch of 8 x 20001, 8 blocks of 640: 14.4 us, with Q = 4 16.4).  Turns
+// are dealt over all rows: a CTA per row left most warps idle where a row has few slices
+// (700 x 8192 x 700 FP8 product with 3: 61.6 us against 58.5).
 constexpr int kQuant = 4;
 
+template <int Q_>
 __global__ void __launch_bounds__(256) quantize_fp8_kernel(const float *__restrict__ Y, int64_t ldy, int64_t rows,
                                                            int32_t b, BlockList blocks,
                                                            __nv_fp8_e4m3 *__restrict__ Q, int64_t ldq,
                                                            float *__restrict__ scales, int64_t lds) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31;
     const int spb = b / 128;                       // slices per block
     const int per_row = blocks.count * spb;
-    for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
-        for (int s0 = warp * kQuant; s0 < per_row; s0 += 8 * kQuant) {
-            float4 v[kQuant];
-            int64_t q0[kQuant];
+    const uint32_t per = (uint32_t)((per_row + Q_ - 1) / Q_);   // warps' turns per row
+    const int64_t total = rows * per, step = (int64_t)gridDim.x * 8;
+    for (int64_t w = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); w < total; w += step) {
+        const int64_t r = total < (int64_t(1) << 32) ? (int64_t)((uint32_t)w / per) : w / per;
+        const int s0 = (int)(w - r * per) * Q_;
+        float4 v[Q_];
+        int64_t q0[Q_];
 #pragma unroll
-            for (int u = 0; u < kQuant; ++u) {
-                const int s = min(s0 + u, per_row - 1);
-                const int bt = s / spb;
-                q0[u] = (int64_t)blocks.idx[bt] * b + (int64_t)(s - bt * spb) * 128;
-                v[u] = __ldcs(reinterpret_cast<const float4 *>(Y + r * ldy + q0[u]) + lane);
-            }
+        for (int u = 0; u < Q_; ++u) {
+            const int s = min(s0 + u, per_row - 1);
+            const int bt = s / spb;
+            q0[u] = (int64_t)blocks.idx[bt] * b + (int64_t)(s - bt * spb) * 128;
+            v[u] = __ldcs(reinterpret_cast<const float4 *>(Y + r * ldy + q0[u]) + lane);
+        }
 #pragma unroll
-            for (int u = 0; u < kQuant; ++u) {
-                if (s0 + u >= per_row) break;
-                float a = fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w)));
+        for (int u = 0; u < Q_; ++u) {
+            if (s0 + u >= per_row) break;
+            float a = fmaxf(fmaxf(fabsf(v[u].x), fabsf(v[u].y)), fmaxf(fabsf(v[u].z), fabsf(v[u].w)));
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-                const int e = fp8_scale_exponent(a);
-                const float inv = ldexpf(1.f, -e);
-                __nv_fp8_e4m3 c[4] = {__nv_fp8_e4m3(v[u].x * inv), __nv_fp8_e4m3(v[u].y * inv),
-                                      __nv_fp8_e4m3(v[u].z * inv), __nv_fp8_e4m3(v[u].w * inv)};
-                *reinterpret_cast<uint32_t *>(Q + r * ldq + q0[u] + 4 * lane) = *reinterpret_cast<const uint32_t *>(c);
-                if (lane == 0) scales[(q0[u] / 128) * lds + r] = ldexpf(1.f, e);   // slice-major
-            }
+            for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+            const int e = fp8_scale_exponent(a);
+            const float inv = ldexpf(1.f, -e);
+            __nv_fp8_e4m3 c[4] = {__nv_fp8_e4m3(v[u].x * inv), __nv_fp8_e4m3(v[u].y * inv),
+                                  __nv_fp8_e4m3(v[u].z * inv), __nv_fp8_e4m3(v[u].w * inv)};
+            *reinterpret_cast<uint32_t *>(Q + r * ldq + q0[u] + 4 * lane) = *reinterpret_cast<const uint32_t *>(c);
+            if (lane == 0) scales[(q0[u] / 128) * lds + r] = ldexpf(1.f, e);   // slice-major
         }
     }
 }
@@ -1024,8 +1031,12 @@ __global__ void __launch_bounds__(256) quantize_fp8_kernel(const float *__restri
 os_status launch_quantize_fp8(const Plan *p, const float *Y, int64_t ldy, int64_t rows, uint64_t block_mask,
                               void *Q, int64_t ldq, float *scales, int64_t lds, cudaStream_t st) {
     const BlockList blocks = mask_to_list(block_mask ? block_mask : ~0ull, p->P);
-    quantize_fp8_kernel<<<(unsigned)(rows < 152 * 64 ? rows : 152 * 64), 256, 0, st>>>(
-        Y, ldy, rows, p->b, blocks, (__nv_fp8_e4m3 *)Q, ldq, scales, lds);
+    const int64_t per_row = (int64_t)blocks.count * (p->b / 128);
+    const bool one = rows * per_row <= 152 * 64;
+    const int64_t ctas = (rows * (one ? per_row : (per_row + kQuant - 1) / kQuant) + 7) / 8;
+    auto k = one ? quantize_fp8_kernel<1> : quantize_fp8_kernel<kQuant>;
+    k<<<(unsigned)(ctas < 152 * 64 ? ctas : 152 * 64), 256, 0, st>>>(Y, ldy, rows, p->b, blocks, (__nv_fp8_e4m3 *)Q, ldq,
+                                                                   scales, lds);
     return check_launch();
 }
 

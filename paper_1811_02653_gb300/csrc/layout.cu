@@ -42,11 +42,12 @@ __global__ void __launch_bounds__(256) select_transpose_kernel(const TI *__restr
     }
 }
 
-// Y = X, eight elements per thread and step (16-byte accesses where kVecX / kVecY: the
-// rows of X / Y start on 16-byte boundaries), threads (x) along a row, (y) and CTAs along the rows.
+// Y = X, eight elements per thread and step (16-byte stores, and loads where kVecX: the
+// rows of Y, of X, start on 16-byte boundaries), threads (x) along a row, (y) and CTAs
+// along the rows.
 // Memory-bound: one element per thread behind a 64-bit division took 46 us for the
 // 4096 x 4096 FP32 -> BF16 cast on GB300 (15 at the copy rate), this takes 14.7.
-template <typename TI, typename TO, bool kVecX, bool kVecY>
+template <typename TI, typename TO, bool kVecX>
 __global__ void __launch_bounds__(256) cast_kernel(const TI *__restrict__ X, int64_t ldx, int64_t rows, int64_t cols,
                                                    TO *__restrict__ Y, int64_t ldy) {
     const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
@@ -67,7 +68,7 @@ __global__ void __launch_bounds__(256) cast_kernel(const TI *__restrict__ X, int
         }
 #pragma unroll
         for (int k = 0; k < 8; ++k) o[k] = from_f<TO>(to_f(a[k]));
-        if (kVecY && whole) {
+        if (whole) {
 #pragma unroll
             for (int k = 0; k < (int)sizeof(o) / 16; ++k)
                 reinterpret_cast<uint4 *>(y)[k] = reinterpret_cast<const uint4 *>(o)[k];
@@ -76,6 +77,28 @@ __global__ void __launch_bounds__(256) cast_kernel(const TI *__restrict__ X, int
             for (int k = 0; k < 8; ++k)
                 if (c + k < cols) y[k] = o[k];
         }
+    }
+}
+
+// The same where the rows of Y do not start on 16-byte boundaries: a warp's lanes take
+// consecutive elements, so that a store still covers whole lines (3000 x 3001 BF16 -> FP32,
+// odd pitches: 27.3 us with eight consecutive elements per thread, 9.1 this way).
+template <typename TI, typename TO>
+__global__ void __launch_bounds__(256) cast_lanes_kernel(const TI *__restrict__ X, int64_t ldx, int64_t rows,
+                                                         int64_t cols, TO *__restrict__ Y, int64_t ldy) {
+    constexpr int U = 8;
+    const int64_t c = (int64_t)blockIdx.x * (U * blockDim.x) + threadIdx.x;
+    if (c >= cols) return;
+    for (int64_t r = (int64_t)blockIdx.y * blockDim.y + threadIdx.y; r < rows; r += (int64_t)gridDim.y * blockDim.y) {
+        const TI *x = X + r * ldx + c;
+        TO *y = Y + r * ldy + c;
+        TI a[U];
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (c + k * blockDim.x < cols) a[k] = x[k * blockDim.x];
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (c + k * blockDim.x < cols) y[k * blockDim.x] = from_f<TO>(to_f(a[k]));
     }
 }
 
@@ -90,16 +113,17 @@ os_status launch_st(const void *X, int64_t ldx, int64_t rows, int64_t ocols, int
 
 template <typename TI, typename TO>
 os_status launch_cast(const void *X, int64_t ldx, int64_t rows, int64_t cols, void *Y, int64_t ldy, cudaStream_t st) {
+    const bool vx = aligned16(X) && (ldx * (int64_t)sizeof(TI)) % 16 == 0;
+    const bool vy = aligned16(Y) && (ldy * (int64_t)sizeof(TO)) % 16 == 0;
+    const bool lanes = !vy;
     const int64_t pieces = (cols + 7) / 8;
-    unsigned tx = 256;
-    while (tx > 1 && (int64_t)tx / 2 >= pieces) tx /= 2;
+    unsigned tx = 256, least = 1;
+    while (lanes && least < 32u && least < cols) least *= 2;
+    while (tx > least && (int64_t)tx / 2 >= pieces) tx /= 2;
     const unsigned ty = 256 / tx;
     const int64_t gy = (rows + ty - 1) / ty;
     const dim3 grid((unsigned)((pieces + tx - 1) / tx), (unsigned)(gy < 16384 ? gy : 16384)), block(tx, ty);
-    const bool vx = aligned16(X) && (ldx * (int64_t)sizeof(TI)) % 16 == 0;
-    const bool vy = aligned16(Y) && (ldy * (int64_t)sizeof(TO)) % 16 == 0;
-    auto k = vx ? (vy ? cast_kernel<TI, TO, true, true> : cast_kernel<TI, TO, true, false>)
-                : (vy ? cast_kernel<TI, TO, false, true> : cast_kernel<TI, TO, false, false>);
+    auto k = lanes ? cast_lanes_kernel<TI, TO> : vx ? cast_kernel<TI, TO, true> : cast_kernel<TI, TO, false>;
     k<<<grid, block, 0, st>>>((const TI *)X, ldx, rows, cols, (TO *)Y, ldy);
     return check_launch();
 }

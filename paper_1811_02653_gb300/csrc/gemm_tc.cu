@@ -666,6 +666,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                 }
             }
         }
+        __syncwarp();         // lanes past the tile's width left the loop early
         cluster_sync_all();   // nobody reads this CTA's shared memory any more
     }
     if (warp == 1) {

@@ -29,6 +29,7 @@
 #include <cstdio>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "group.cuh"
@@ -95,7 +96,10 @@ struct Cfg {
     // in TMEM and the epilogue adds the chunks in FP32 registers, so the
     // accumulation error does not grow with K.  Otherwise one chunk per tile.
     static constexpr int CHUNK_KB = kKind == Kind::Tf32x3 ? 8 : (1 << 30);
-    // fewest K steps per CTA of a split tile (0: never split)
+    // fewest K steps per CTA of a split tile (0: never split) and of the tile: FP8 tiles of
+    // three steps take 9.3 us in two parts and 8.6 whole (500 x 700; of four 9.4 and 8.9, but
+    // 1 x 479 6.8 and 7.3)
+    static constexpr int SPLIT_FROM_KB = kKind == Kind::Fp8 ? 4 : 0;
     static constexpr int MIN_SPLIT_KB = kKind == Kind::Tf32x3 ? 4 : kKind == Kind::Fp8 ? 2 : 0;
     static_assert(!FP8 || (BN <= 240 && 2 * SF_GAP_SLOTS >= STAGES), "FP8 scale slots do not fit in TMEM");
     static_assert(BN % 32 == 0 && BN <= 256, "tile width");
@@ -182,40 +186,71 @@ __device__ __forceinline__ void tile_coords(int t, int tiles_m, int tiles_n, int
 // grouped launch of 16 uneven products 861 -> 779, the FP8 product of 8192^3
 // (16-byte stores, beside the next tile's MMAs) 514 -> 472.
 // The odd pitch keeps both the column writes and the row reads free of conflicts.
+// kBatch: eight values per lane are read from the piece before they are stored (the
+// compiler cannot tell the two apart and waits for every read in turn): what thin and
+// short tiles wait for (31 x 2121 FP8, K = 512: 11.3 -> 9.1 us).  Not where the registers
+// are all taken (FP16 planes: 8192 x 32768 x 8192 would take 25 us longer).
+template <bool kBatch>
 __device__ __forceinline__ void store_piece(float *buf, const float *v, float alpha, float beta, float *C,
                                             int64_t ldc, int64_t r0, int64_t m, int64_t cb, int64_t l, bool vec_ok,
                                             int lane) {
+    if (r0 >= m || cb >= l) return;   // nothing of the piece lies in C
     __syncwarp();   // the previous piece has been read
 #pragma unroll
     for (int u = 0; u < 32; ++u) buf[lane * kEpiPitch + u] = alpha * v[u];
     __syncwarp();
     if (vec_ok && cb + 32 <= l) {
         // 4 rows per instruction, 8 lanes of 16 bytes each
+        constexpr int NV = kBatch ? 2 : 1;
         const int rr = lane >> 3, cc = (lane & 7) * 4;
         float *dst = C + (r0 + rr) * ldc + cb + cc;
 #pragma unroll
-        for (int t = 0; t < 8; ++t, dst += 4 * ldc) {
-            const float *src = buf + (4 * t + rr) * kEpiPitch + cc;
-            float4 o = make_float4(src[0], src[1], src[2], src[3]);
-            if (r0 + 4 * t + rr < m) {
-                if (beta != 0.f) {
-                    const float4 old = *reinterpret_cast<const float4 *>(dst);
-                    o.x = fmaf(beta, old.x, o.x);
-                    o.y = fmaf(beta, old.y, o.y);
-                    o.z = fmaf(beta, old.z, o.z);
-                    o.w = fmaf(beta, old.w, o.w);
+        for (int t0 = 0; t0 < 8; t0 += NV) {
+            float4 o[NV];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const float *src = buf + (4 * (t0 + k) + rr) * kEpiPitch + cc;
+                o[k] = make_float4(src[0], src[1], src[2], src[3]);
+            }
+#pragma unroll
+            for (int k = 0; k < NV; ++k, dst += 4 * ldc) {
+                if (r0 + 4 * (t0 + k) + rr < m) {
+                    if (beta != 0.f) {
+                        const float4 old = *reinterpret_cast<const float4 *>(dst);
+                        o[k].x = fmaf(beta, old.x, o[k].x);
+                        o[k].y = fmaf(beta, old.y, o[k].y);
+                        o[k].z = fmaf(beta, old.z, o[k].z);
+                        o[k].w = fmaf(beta, old.w, o[k].w);
+                    }
+                    *reinterpret_cast<float4 *>(dst) = o[k];
                 }
-                *reinterpret_cast<float4 *>(dst) = o;
             }
         }
     } else if (cb + lane < l) {
         float *dst = C + r0 * ldc + cb + lane;
+        if constexpr (kBatch) {
+            const int rows = m - r0 < 32 ? (int)(m - r0) : 32;
+#pragma unroll 1
+            for (int t0 = 0; t0 < rows; t0 += 8) {
+                float o[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) o[k] = buf[(t0 + k) * kEpiPitch + lane];
+#pragma unroll
+                for (int k = 0; k < 8; ++k, dst += ldc) {
+                    if (t0 + k < rows) {
+                        if (beta != 0.f) o[k] = fmaf(beta, *dst, o[k]);
+                        *dst = o[k];
+                    }
+                }
+            }
+        } else {
 #pragma unroll 8
-        for (int t = 0; t < 32; ++t, dst += ldc) {
-            if (r0 + t < m) {
-                float o = buf[t * kEpiPitch + lane];
-                if (beta != 0.f) o = fmaf(beta, *dst, o);
-                *dst = o;
+            for (int t = 0; t < 32; ++t, dst += ldc) {
+                if (r0 + t < m) {
+                    float o = buf[t * kEpiPitch + lane];
+                    if (beta != 0.f) o = fmaf(beta, *dst, o);
+                    *dst = o;
+                }
             }
         }
     }
@@ -570,7 +605,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                         dst[u] = make_float4(val[4 * u], val[4 * u + 1], val[4 * u + 2], val[4 * u + 3]);
                     return;
                 }
-                store_piece(buf, val, j.alpha, j.beta, j.C, j.ldc, r0, j.m, c0 + ch * 32, j.l, vec_ok, lane);
+                store_piece<true>(buf, val, j.alpha, j.beta, j.C, j.ldc, r0, j.m, c0 + ch * 32, j.l, vec_ok, lane);
             };
             if constexpr (C::CHUNK_KB < (1 << 30)) {
                 // chunked accumulation: running FP32 sum of the tile row in registers
@@ -604,6 +639,7 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
                 if (!__all_sync(0xffffffffu, mbar_wait(&tmem_full[a], aphase, abort, wait_ns))) break;
                 tc_fence_after();
                 for (int ch = 0; ch < BN / 32; ++ch) {
+                    if (r0 >= j.m || c0 + ch * 32 >= j.l) break;   // nothing of it lies in C
                     uint32_t v[32];
                     if (j.num_kb > 0) {
                         tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) +
@@ -626,46 +662,63 @@ gemm_masked_tc_kernel(const __grid_constant__ CUtensorMap tmap_a0, const __grid_
         cluster_sync_all();   // every partial tile is written
         const TileJob j = job(t_first);
         const bool vec_ok = ((reinterpret_cast<uintptr_t>(j.C) & 15u) == 0) && (j.ldc % 4 == 0);
-        const int rows = BM / g.split;
+        constexpr int WARPS = C::THREADS / 32;
         const uint32_t part = smem_u32(tiles);
-        for (int q = warp; q < rows; q += C::THREADS / 32) {
-            const int row = rank * rows + q;
-            const int64_t r = (int64_t)j.tm * BM + row;
-            if (r >= j.m) break;
-            for (int c = 4 * lane; c < BN; c += 128) {
-                const uint32_t at = part + 4u * (uint32_t)(row * PART_PITCH + c);
-                float4 v[8];
+        // a warp's rows 8 / S at a time: eight loads per lane in flight whatever the split
+        // (one row at a time the two CTAs of a split tile took 2.5 us here)
+        auto add_parts = [&](auto ss) {
+            constexpr int S = decltype(ss)::value, R = 8 / S, rows = BM / S;
+            for (int q = warp; q < rows; q += R * WARPS) {
+                const int row = rank * rows + q;
+                const int64_t r = (int64_t)j.tm * BM + row;
+                if (r >= j.m) break;
+                for (int c = 4 * lane; c < BN; c += 128) {
+                    const int64_t cb = (int64_t)j.tn * BN + c;
+                    if (cb >= j.l) break;
+                    float4 v[R][S];
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    if (k < g.split) v[k] = ld_cluster_v4(cluster_addr_of(at, (uint32_t)k));
-                float4 o = v[0];
+                    for (int i = 0; i < R; ++i) {
+                        // rows past the CTA's last one: the last one again
+                        const int at = row + (q + i * WARPS < rows ? i * WARPS : rows - 1 - q);
 #pragma unroll
-                for (int k = 1; k < 8; ++k)
-                    if (k < g.split) {
-                        o.x += v[k].x;
-                        o.y += v[k].y;
-                        o.z += v[k].z;
-                        o.w += v[k].w;
+                        for (int k = 0; k < S; ++k)
+                            v[i][k] = ld_cluster_v4(
+                                cluster_addr_of(part + 4u * (uint32_t)(at * PART_PITCH + c), (uint32_t)k));
                     }
-                const int64_t cb = (int64_t)j.tn * BN + c;
-                float x[4] = {j.alpha * o.x, j.alpha * o.y, j.alpha * o.z, j.alpha * o.w};
-                float *dst = j.C + r * j.ldc + cb;
-                if (vec_ok && cb + 4 <= j.l) {
-                    if (j.beta != 0.f) {
-                        const float4 old = *reinterpret_cast<const float4 *>(dst);
-                        x[0] = fmaf(j.beta, old.x, x[0]);
-                        x[1] = fmaf(j.beta, old.y, x[1]);
-                        x[2] = fmaf(j.beta, old.z, x[2]);
-                        x[3] = fmaf(j.beta, old.w, x[3]);
-                    }
-                    *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
-                } else {
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (cb + u < j.l) dst[u] = j.beta != 0.f ? fmaf(j.beta, dst[u], x[u]) : x[u];
+                    for (int i = 0; i < R; ++i) {
+                        if (q + i * WARPS >= rows || r + i * WARPS >= j.m) break;
+                        float4 o = v[i][0];
+#pragma unroll
+                        for (int k = 1; k < S; ++k) {
+                            o.x += v[i][k].x;
+                            o.y += v[i][k].y;
+                            o.z += v[i][k].z;
+                            o.w += v[i][k].w;
+                        }
+                        float x[4] = {j.alpha * o.x, j.alpha * o.y, j.alpha * o.z, j.alpha * o.w};
+                        float *dst = j.C + (r + i * WARPS) * j.ldc + cb;
+                        if (vec_ok && cb + 4 <= j.l) {
+                            if (j.beta != 0.f) {
+                                const float4 old = *reinterpret_cast<const float4 *>(dst);
+                                x[0] = fmaf(j.beta, old.x, x[0]);
+                                x[1] = fmaf(j.beta, old.y, x[1]);
+                                x[2] = fmaf(j.beta, old.z, x[2]);
+                                x[3] = fmaf(j.beta, old.w, x[3]);
+                            }
+                            *reinterpret_cast<float4 *>(dst) = make_float4(x[0], x[1], x[2], x[3]);
+                        } else {
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                if (cb + u < j.l) dst[u] = j.beta != 0.f ? fmaf(j.beta, dst[u], x[u]) : x[u];
+                        }
+                    }
                 }
             }
-        }
+        };
+        if (g.split == 2) add_parts(std::integral_constant<int, 2>());
+        else if (g.split == 4) add_parts(std::integral_constant<int, 4>());
+        else add_parts(std::integral_constant<int, 8>());
         __syncwarp();         // lanes past the tile's width left the loop early
         cluster_sync_all();   // nobody reads this CTA's shared memory any more
     }
@@ -919,7 +972,7 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
                     for (int u = 0; u < 32; ++u) v[u] = 0u;
                 }
                 const int64_t cb = c0 + ch * 32;
-                store_piece(buf, reinterpret_cast<const float *>(v), alpha, g.beta, g.C, g.ldc, r - lane, g.m, cb, g.l,
+                store_piece<true>(buf, reinterpret_cast<const float *>(v), alpha, g.beta, g.C, g.ldc, r - lane, g.m, cb, g.l,
                             vec_ok, lane);
                 if (r < g.m) {
                     if (g.sym && (tm >> 1) != tn) {
@@ -1189,7 +1242,7 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                 float *tv = total + ch * 32;
 #pragma unroll
                 for (int u = 0; u < 32; ++u) tv[u] = tv[u] * sa * __shfl_sync(0xffffffffu, sb, u);
-                store_piece(buf, tv, g.alpha, g.beta, g.C, g.ldc, r0, g.m, cb, g.l, vec_ok, lane);
+                store_piece<false>(buf, tv, g.alpha, g.beta, g.C, g.ldc, r0, g.m, cb, g.l, vec_ok, lane);
             }
         }
     }
@@ -1467,7 +1520,7 @@ gemm_pair_fp8_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
             for (int ch = 0; ch < BN / 32; ++ch) {
                 uint32_t v[32];
                 tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * 256 + ch * 32), v);
-                store_piece(buf, reinterpret_cast<const float *>(v), g.alpha, g.beta, g.C, g.ldc, r0, g.m, c0 + ch * 32,
+                store_piece<true>(buf, reinterpret_cast<const float *>(v), g.alpha, g.beta, g.C, g.ldc, r0, g.m, c0 + ch * 32,
                             g.l, vec_ok, lane);
             }
             tc_fence_before();
@@ -1608,6 +1661,7 @@ int split_of(int64_t tiles, int num_kb, int min_kb) {
             }
         }
     });
+    if (num_kb < C::SPLIT_FROM_KB) return 1;
     for (int i = 3; i >= 1; --i) {
         const int S = 1 << i, per = (num_kb + S - 1) / S;
         if (tiles <= resident[i] && per >= min_kb && (S - 1) * per < num_kb) return S;

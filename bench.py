@@ -385,6 +385,21 @@ def run_ours(args):
     h2d = A_h.numel() * 4 + B_h.numel() * 4
     d2h = C_h.numel() * 4
 
+    # the product as a caller makes it, one oversketch_matmul on the device operands (an FP32
+    # product of this size runs on FP16 planes there, not as the three calls' 3xTF32)
+    def product_ms(f, ws_f, reps):
+        ops.matmul(p, A, B, w.mask, f, C=C, workspace=ws_f)
+        torch.cuda.synchronize()
+        p0, p1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        p0.record(stream)
+        for _ in range(reps):
+            ops.matmul(p, A, B, w.mask, f, C=C, workspace=ws_f)
+        p1.record(stream)
+        torch.cuda.synchronize()
+        return _max_over_ranks(p0.elapsed_time(p1) / reps, world)
+
+    matmul_ms = product_ms(gd, ws_mm, max(3, min(args.steps, 10)))
+
     # ---- the other GEMM dtypes on the same inputs (same three calls, own sketch buffers) ----
     forms = {}
     if not args.no_forms:
@@ -403,7 +418,7 @@ def run_ours(args):
             ms_f, per_f, _ = _time_phases(phases_f, max(3, min(args.steps, 10)), 2, world, sample_clocks=False)
             forms[f] = {"ms_per_step": ms_f, "tflops": _job_value(2.0 * w.m * w.n * w.l, ms_f, world),
                         "phases_ms": {k_: round(v_, 4) for k_, v_ in per_f.items()},
-                        "sketch_dtype": sf}
+                        "sketch_dtype": sf, "matmul_ms": product_ms(f, ws_f, 3)}
             del Af, Bf, asf, bsf, ws_f
         torch.cuda.synchronize()
 
@@ -535,7 +550,7 @@ def run_ours(args):
                     "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms},
             # pack + gather (left), gather (right), GEMM; FP8 adds the two quantisation passes
             "gpu_launches": (6 if sd == "fp8" else 4) * args.steps, "clocks": clk, "error": err, "exact_gemm": exact,
-            "forms": forms,
+            "matmul_ms": matmul_ms, "forms": forms,
             "plan_ms": _plan_record(plan_s, plan_dev)}
     if rank == 0:
         print(json.dumps(line), flush=True)

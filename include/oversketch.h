@@ -289,8 +289,9 @@ OS_API os_status oversketch_gemm_masked_blocks(oversketch_plan_t plan, const voi
 /* -------------------------------------------------------------------------
  * The whole product (*): left sketch, right sketch, masked GEMM.  An OS_F32 product
  * sketches in FP32; large ones then split the sums into FP16 planes with one
- * power-of-two scale per row (dropped terms 2^-24 of the row), unless a row's range
- * does not suit them (decided on the device), others run as 3xTF32.
+ * power-of-two scale per row (2^-23 of each entry, 2^-21 of the smallest; the
+ * few below 2^-30 of their row's largest are added in FP32), unless the operands'
+ * range does not suit them (decided on the device), others run as 3xTF32.
  */
 typedef struct {
     os_dtype gemm_dtype;      /* OS_F32, OS_BF16 or OS_FP8E4M3               */

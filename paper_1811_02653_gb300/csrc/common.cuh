@@ -56,8 +56,10 @@ struct SplitSide {
 // What the split leaves for the launches after it, in the product's scratch: flag, set
 // when the planes do not suit the operands (the product then runs on TF32 planes), and
 // the entries left out of the planes: their count, then row (bit 31: of B) and column.
-// 2048 entries: operands of random sums have a few, heavy-tailed ones some hundred.
-constexpr unsigned int kSplitLost = 2048;
+// Operands of random sums have one or none, an interior-point matrix of some thousand
+// rows hundreds to thousands.
+constexpr unsigned int kSplitLost = 16384;     // entries at most, 2048 of them in one row
+constexpr unsigned int kSplitLostRow = 2048;
 struct SplitCtl {
     unsigned int flag, lost, pad[2];
     uint2 entry[kSplitLost];

@@ -39,7 +39,7 @@ namespace osk {
 
 // implemented in split.cu
 os_status launch_split_f16(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
-                           SplitCtl *ctl, cudaStream_t st);
+                           SplitCtl *ctl, unsigned int most, cudaStream_t st);
 os_status launch_split_correct(const SplitSide &a, const SplitSide &b, int64_t ld, int32_t blk, const BlockList &kept,
                                const SplitCtl *ctl, float alpha, float *C, int64_t ldc, int64_t l, cudaStream_t st);
 
@@ -1006,11 +1006,11 @@ gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_c
 
 // ---------------------------------------------------------------------------
 // FP32-accuracy masked GEMM on FP16 planes (split.cu), CTA pairs:
-//   A~ B~ = hi.hi + (hi.lo + lo.hi) / 2048        (lo.lo, up to 2^-22 of the terms, dropped)
+//   A~ B~ = hi.hi + (hi.lo + lo.hi) / 4096        (lo.lo, 2^-22 .. 2^-20 of the terms, dropped)
 // The organisation of gemm_pair_bf16_kernel with 256 x 160 tiles and two kinds of
 // accumulators: hi.hi in chunks of K = 256, double-buffered, which the epilogue
 // adds in FP32 registers (the tensor core's FP32 accumulation truncates, so its
-// error must not grow with K), and the 2048 times smaller cross terms in one
+// error must not grow with K), and the 4096 times smaller cross terms in one
 // accumulator over the whole K, which their truncation never reaches.  3 x 160
 // columns is what TMEM holds of the two.  Bound by the tensor pipe: a K step of 64
 // is 12 MMAs (960 tensor clocks) on 52 KB per CTA, 136 bytes of shared memory per clock.
@@ -1217,7 +1217,7 @@ gemm_pair_f16x3_kernel(const __grid_constant__ CUtensorMap tmap_ah, const __grid
                         tmem_ld_32x32b_x32(lanes + (uint32_t)(C::CROSS + ch * 32), v);
 #pragma unroll
                         for (int u = 0; u < 32; ++u)
-                            total[ch * 32 + u] = fmaf(0x1p-11f, __uint_as_float(v[u]), total[ch * 32 + u]);
+                            total[ch * 32 + u] = fmaf(0x1p-12f, __uint_as_float(v[u]), total[ch * 32 + u]);
                     }
                     tc_fence_before();
                     mbar_arrive_cluster(cross_cl);
@@ -1934,6 +1934,9 @@ os_status gemm_bf16_mn(const void *A, int64_t lda, bool a_mn, const void *B, int
     return launch_pair_bf16_mn(A, lda, a_mn, B, ldb, b_mn, m, l, K, alpha, 0.0f, C, ldc, mn_b, remap, kept, P, st);
 }
 
+double tf32x3_us(int64_t m, int64_t l, int64_t K);
+double f16x3_us(int64_t m, int64_t l, int64_t K);
+
 // The FP32-accuracy product from FP32 sums on FP16 planes (gemm_pair_f16x3_kernel):
 // split both operands, multiply, add the products of the entries that the split left out
 // of the planes, and behind the split's flag the 3xTF32 product of the same sums for
@@ -1946,7 +1949,11 @@ os_status gemm_masked_f16x3(const Plan *p, const SplitSide &a, const SplitSide &
     const int64_t m = a.rows, z = (int64_t)p->P * p->b;
     if (p->b % C::BKE != 0 || z >= (int64_t(1) << 31)) return OS_ERR_UNSUPPORTED;
     if (!aligned16(a.sums) || !aligned16(bs.sums) || ld % 8 != 0) return OS_ERR_INVALID_ARG;
-    OSK_TRY(launch_split_f16(a, b, ld, p->b, kept, ctl, st));
+    // as many listed entries as cost no more than 3xTF32 would
+    constexpr double kListedUs = 1.1e-5;   // per entry and element of C it adds to (split.cu)
+    const int64_t K = (int64_t)kept.count * p->b;
+    const double most = (tf32x3_us(m, l, K) - f16x3_us(m, l, K)) / (kListedUs * (double)(b.rows ? (m > l ? m : l) : 2 * m));
+    OSK_TRY(launch_split_f16(a, b, ld, p->b, kept, ctl, most < 256.0 ? 256u : most < 16384.0 ? (unsigned int)most : 16384u, st));
     GemmArgs g;
     std::memset(&g, 0, sizeof(g));
     g.m = m;

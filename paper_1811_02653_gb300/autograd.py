@@ -26,8 +26,9 @@ from . import ops
 def _sketches(X, G, plan, mask):
     """The BF16 sketches of both operands (kept blocks), one packing workspace for the
     two: small layers are bound by the host, a tensor allocation is 2 - 7 us there."""
-    ops._rowmajor(X, "A")   # before the shapes are read
-    ops._rowmajor(G, "B")
+    if X.dim() != 2 or G.dim() != 2:   # refused by name before the shapes are read
+        ops._rowmajor(X, "A")
+        ops._rowmajor(G, "B")
     ws = torch.empty(max(ops.sketch_workspace(plan, X.shape[0], X.dtype), ops.sketch_workspace(plan, G.shape[1], G.dtype)),
                      dtype=torch.uint8, device=X.device)
     At, _ = ops.sketch_left(plan, X, "bf16", block_mask=mask, workspace=ws)

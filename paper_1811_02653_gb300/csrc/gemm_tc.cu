@@ -1631,8 +1631,8 @@ cudaError_t launch_clusters(Kern kern, unsigned cluster, unsigned grid, int thre
 // behind a serial chain of K steps: as many as are resident at once (clusters do not
 // straddle GPCs: 76, 36 and 15 of 2, 4 and 8 CTAs; 16 clusters of 8 took two rounds,
 // slower than 16 of 4), with at least min_kb K steps each, all of them with some.
-// us for the 3xTF32 GEMM on GB300, whole -> split: 512 x 512, K = 1024 25 -> 12.7;
-// 512 x 512, 4096 78 -> 25.7; 300 x 300, 8192 150 -> 26.4; 1024 x 1024, 4096 80 -> 45.6.
+// us for the 3xTF32 GEMM on GB300, whole -> split: 500 x 700, K = 1024 23.3 -> 11.0;
+// 300 x 300, 2048 40.8 -> 10.8; 128 x 128, 4096 78 -> 15.2; 1000 x 700, 4096 79 -> 41.9.
 template <class C>
 int split_of(int64_t tiles, int num_kb, int min_kb) {
     static std::once_flag once;

@@ -28,8 +28,9 @@
 //   A row with more nonzeros in some warp's share than a region holds is left to the
 //   flushing kernel: its first kept output gets a marker value.
 //   Bound by HBM and instruction issue together.  4096 x 2^20 FP32 at 1 % (17.2 GB,
-//   2.54 ms at the copy rate), 6 kept blocks of 4096, on GB300: 3.97 ms (5.47 with
-//   one row at a time and 1024 threads; the compaction alone 2.71; 2.84 ms at 0.3 %).
+//   2.54 ms at the copy rate), 6 kept blocks of 4096, with column scales, on GB300: 3.73
+//   ms (3.97 before regions of a size known at compile time; 5.47 with an earlier kernel of
+//   one row at a time; the compaction alone 2.71).
 //   Routing both rows at once, with bucket tables for each group, took 4.28 ms.
 //   What the routing's instructions cost decides: predicated accesses in place of
 //   branches around them, and sums without branches, gave 4.80 -> 4.02; buckets
